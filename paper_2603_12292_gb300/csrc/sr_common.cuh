@@ -14,6 +14,7 @@ struct sr_ctx {
   // growable device workspace (scratch for partial sums, queues, stacks)
   char *ws = nullptr;
   size_t ws_bytes = 0;
+  bool ws_fixed = false;  // the workspace is not the context's own: it never grows
   // small permanent device block: [0] latched error word, [1..] spare
   unsigned *dev_words = nullptr;
   char msg[512] = {0};

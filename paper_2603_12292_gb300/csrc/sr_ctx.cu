@@ -45,6 +45,7 @@ sr_status allow_dynamic_smem(sr_ctx *ctx, const void *kernel) {
 
 sr_status ensure_workspace(sr_ctx *ctx, size_t bytes) {
   if (bytes <= ctx->ws_bytes) return SR_OK;
+  if (ctx->ws_fixed) return fail(ctx, SR_ENOMEM, "workspace of %zu bytes needed (have %zu)", bytes, ctx->ws_bytes);
   if (stream_capturing(ctx))
     return fail(ctx, SR_ENOMEM,
                 "workspace of %zu bytes needed during stream capture (have %zu); "

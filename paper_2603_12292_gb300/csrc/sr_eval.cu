@@ -41,14 +41,12 @@
 
 #include "sr_common.cuh"
 #include "sr_interp.cuh"
+#include "sr_vm.cuh"
 
 namespace sr {
 namespace {
 
 constexpr int WARPS = 8;        // warps per CTA (measured best of 4, 8, 16 warps per CTA)
-constexpr int CPL = 8;          // cases per lane per dispatched instruction (two float4)
-constexpr int STEP = 32 * CPL;  // cases per warp step
-constexpr int SLOT_BYTES = 32 * CPL * 4;  // one stack slot of a warp: [2][32 lanes] float4
 constexpr int PSTRIDE = 8;      // doubles per partial record
 // Calls of at least this many cases and programs read the unary transforms
 // of the variables from a table (sr_set_transforms' automatic mode); below
@@ -101,35 +99,39 @@ struct EvalParams {
   long long ldy;
   int warp_bytes;          // shared memory per warp
   int slots;               // stack slots per warp
-  int deep;                // 1: this launch is the pass of the NCODE_DEEP programs
+  int pass;                // Pass: the programs this launch takes
   int score_M;             // Beagle scores: the maximum score per case
   const int32_t *abort;    // sr_set_abort_flag (or NULL)
   unsigned *err;           // the context's latched error word
   int xform = 0;           // >= 1: X is the variable table of this depth (DecodeArgs::xform)
+  const float *Xsrc = nullptr;  // rows to copy into X (the caller's X, not laid out for 256-bit loads), or NULL
+  long long ldsrc = 0;
   uint8_t *xneed = nullptr;  // the transforms some program reads
 };
 
-__host__ __device__ inline int code_smem_bytes(int Lmax) { return ((Lmax * 8 + 15) / 16) * 16; }
+// a program's code and its end marker
+__host__ __device__ inline int code_smem_bytes(int Lmax) { return (((Lmax + 1) * 8 + 15) / 16) * 16; }
 
 __host__ __device__ inline int warp_smem_bytes(int slots, int Lmax) {
   // stack slots | decoded code (8 bytes per token)
   return slots * SLOT_BYTES + code_smem_bytes(Lmax);
 }
 
-// Stack slots of the main evaluation passes: as many as fit smem_target(minb),
-// at most slots_for(Lmax) and at least min(slots_for(Lmax), 4).  Programs of
-// up to 256 tokens, random or evolved, rarely need more than 4 (Sethi-Ullman
-// order) while slots_for(256) = 7 would leave room for only 3 CTAs per SM;
-// the few that need more than the main passes give (NCODE_DEEP) run in a
-// third pass with slots_for(Lmax) slots.
-__host__ __device__ inline int shallow_slots(int Lmax, int minb) {
+// Stack slots of the main evaluation passes: as many as fit smem_target(minb)
+// beside `code` bytes of code, at most slots_for(Lmax) and at least
+// min(slots_for(Lmax), 4).  Programs of up to 256 tokens, random or evolved,
+// rarely need more than 4 (Sethi-Ullman order) while slots_for(256) = 7 would
+// leave room for only 3 CTAs per SM; the few that need more than the main
+// passes give (NCODE_DEEP) run in a third pass with slots_for(Lmax) slots.
+__host__ __device__ inline int fit_slots(int Lmax, int minb, int code) {
   const int full = slots_for(Lmax), lo = full < 4 ? full : 4;
-  const int s = (smem_target(minb) / WARPS - code_smem_bytes(Lmax)) / SLOT_BYTES;
+  const int s = (smem_target(minb) / WARPS - code) / SLOT_BYTES;
   return s < lo ? lo : (s > full ? full : s);
 }
+__host__ __device__ inline int shallow_slots(int Lmax, int minb) { return fit_slots(Lmax, minb, code_smem_bytes(Lmax)); }
 
 // 5 CTAs per SM where they fit with at least min(slots_for(Lmax), 4) slots
-// (Lmax <= 200), else 4.
+// (Lmax <= 198), else 4.
 inline int minb_for(int Lmax) {
   return WARPS * warp_smem_bytes(shallow_slots(Lmax, 5), Lmax) <= smem_target(5) ? 5 : 4;
 }
@@ -141,16 +143,23 @@ inline int eval_minb(int Lmax, int tuned) {
   return minb_for(Lmax);
 }
 
+// The CTAs per SM that the cases per work item are chosen by: those of a warp
+// with its stack slots and 8 bytes of code per token (no end marker).  The
+// FP32 sums of a program follow its case chunks, so this rule is part of the
+// results and stays as it is whatever the kernels take.
+inline int chunk_ctas(int Lmax, int minb) {
+  const int code = ((Lmax * 8 + 15) / 16) * 16;
+  const int smem = WARPS * (fit_slots(Lmax, minb, code) * SLOT_BYTES + code);
+  const int fit = 233472 / (smem + 1024);
+  return fit < minb ? fit : minb;
+}
+inline int chunk_minb(int Lmax, int tuned) {  // eval_minb by the same rule
+  const int code = ((Lmax * 8 + 15) / 16) * 16;
+  const bool five = WARPS * (fit_slots(Lmax, 5, code) * SLOT_BYTES + code) <= smem_target(5);
+  return tuned == 4 || !five ? 4 : 5;
+}
+
 // ---------------------------------------------------------------- operators
-#define MAP4(f, v) make_float4(f((v).x), f((v).y), f((v).z), f((v).w))
-#define ZIP4(f, a, b) make_float4(f((a).x, (b).x), f((a).y, (b).y), f((a).z, (b).z), f((a).w, (b).w))
-
-__device__ __forceinline__ float f_add(float a, float b) { return a + b; }
-__device__ __forceinline__ float f_sub(float a, float b) { return a - b; }
-__device__ __forceinline__ float f_mul(float a, float b) { return a * b; }
-__device__ __forceinline__ float f_sq(float x) { return x * x; }
-
-__device__ __forceinline__ float4 splat(float c) { return make_float4(c, c, c, c); }
 __device__ __forceinline__ float4 ldx4(const float *p) {
   return __ldg(reinterpret_cast<const float4 *>(p));
 }
@@ -182,10 +191,27 @@ __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_s
   return a;
 }
 
-// one warp per program, scratch in shared memory (decode_warp)
+// Copies X's rows (nvars x N, row stride ldsrc) into rows of ldx floats that
+// start on 32-byte boundaries, so that the interpreter reads a lane's 8 cases
+// with one load.  Blocks of STAGE_CASES cases of one row.
+constexpr int STAGE_CASES = 2048;
+__host__ __device__ inline int stage_blocks(int nvars, int N) { return nvars * ((N + STAGE_CASES - 1) / STAGE_CASES); }
+__device__ void stage_rows(const EvalParams &p, int block) {
+  const int per_row = (p.N + STAGE_CASES - 1) / STAGE_CASES;
+  const int j = block / per_row, end = min(p.N, (block % per_row + 1) * STAGE_CASES);
+  const float *src = p.Xsrc + (size_t)j * p.ldsrc;
+  float *dst = const_cast<float *>(p.X) + (size_t)j * p.ldx;
+  for (int i = (block % per_row) * STAGE_CASES + threadIdx.x * 4; i < end; i += blockDim.x * 4)
+    *reinterpret_cast<float4 *>(dst + i) = ldx4(src + i);  // i + 3 < both strides: multiples of 4, >= N
+}
+
+// one warp per program, scratch in shared memory (decode_warp); the blocks
+// after those copy X where it is not laid out for 256-bit loads
 __global__ void decode_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  decode_warp(decode_args(p, p.slots, p.queue + 4), p.P, dsm);
+  const int dblocks = (p.P + DECODE_WARPS - 1) / DECODE_WARPS;
+  if ((int)blockIdx.x >= dblocks) stage_rows(p, blockIdx.x - dblocks);
+  else decode_warp(decode_args(p, p.slots, p.queue + 4), p.P, dsm);
 }
 
 // The variable table of an evaluation with transforms (DecodeArgs::xform):
@@ -219,186 +245,6 @@ __global__ void __launch_bounds__(XF_THREADS)
   if (u >= 0)
     x = make_float4(fold_op(u, x.x, 0.f), fold_op(u, x.y, 0.f), fold_op(u, x.z, 0.f), fold_op(u, x.w, 0.f));
   *reinterpret_cast<float4 *>(xt + (size_t)r * ldxt + c) = x;
-}
-
-// ---------------------------------------------------------------- interpreter
-// CPL = 8 cases per lane: the value on top of the stack is two float4 (a: the
-// lane's cases 0-3, b: cases 4-7); a stack slot holds the same for every
-// lane as [slot][half][lane] float4, so each 128-bit access of a warp covers
-// 512 contiguous bytes (no bank conflicts).
-struct V8 {
-  float4 a, b;
-};
-
-__device__ __forceinline__ V8 splat8(float c) {
-  V8 r;
-  r.a = splat(c);
-  r.b = r.a;
-  return r;
-}
-#define MAP8(f, v) V8{MAP4(f, (v).a), MAP4(f, (v).b)}
-#define ZIP8(f, p, q) V8{ZIP4(f, (p).a, (q).a), ZIP4(f, (p).b, (q).b)}
-
-__device__ __forceinline__ V8 ld8(const char *stk, uint32_t off) {
-  V8 r;
-  r.a = *reinterpret_cast<const float4 *>(stk + off);
-  r.b = *reinterpret_cast<const float4 *>(stk + off + 32 * 16);
-  return r;
-}
-__device__ __forceinline__ void st8(char *stk, uint32_t off, const V8 &v) {
-  *reinterpret_cast<float4 *>(stk + off) = v.a;
-  *reinterpret_cast<float4 *>(stk + off + 32 * 16) = v.b;
-}
-__device__ __forceinline__ V8 ldX8(const float *xa, const float *xb, uint32_t off) {
-  return V8{ldx4(xa + off), ldx4(xb + off)};
-}
-
-#ifndef SR_MATH_UNROLL
-#define SR_MATH_UNROLL 8
-#endif
-constexpr int MATH_UNROLL = SR_MATH_UNROLL;
-// The costly operators (the FP32 math library routines and the quotient)
-// live out of line, one copy each, so the interpreter's dispatch loop stays
-// small enough for the instruction cache; inside, SR_MATH_UNROLL values are
-// in flight at a time.  Measured on the 4096 x 100,000 mixed population:
-// everything inlined ~1,450 GPop/s, out of line with 4 in flight ~1,530,
-// with 8 in flight ~2,200.
-struct FSin { __device__ __forceinline__ float operator()(float x) const { return f_sin(x); } };
-struct FCos { __device__ __forceinline__ float operator()(float x) const { return f_cos(x); } };
-struct FExp { __device__ __forceinline__ float operator()(float x) const { return op_exp(x); } };
-struct FLog { __device__ __forceinline__ float operator()(float x) const { return op_log(x); } };
-struct FSqrt { __device__ __forceinline__ float operator()(float x) const { return f_sqrt(x); } };
-struct FInv { __device__ __forceinline__ float operator()(float x) const { return op_inv(x); } };
-struct FTan { __device__ __forceinline__ float operator()(float x) const { return f_tan(x); } };
-struct FAsin { __device__ __forceinline__ float operator()(float x) const { return f_asin(x); } };
-struct FAcos { __device__ __forceinline__ float operator()(float x) const { return f_acos(x); } };
-struct FAtan { __device__ __forceinline__ float operator()(float x) const { return f_atan(x); } };
-struct FTanh { __device__ __forceinline__ float operator()(float x) const { return f_tanh(x); } };
-
-template <typename F>
-__device__ __forceinline__ V8 map8_unrolled(V8 v, F f) {
-  float t[8] = {v.a.x, v.a.y, v.a.z, v.a.w, v.b.x, v.b.y, v.b.z, v.b.w};
-#pragma unroll MATH_UNROLL
-  for (int i = 0; i < 8; ++i) t[i] = f(t[i]);
-  return V8{make_float4(t[0], t[1], t[2], t[3]), make_float4(t[4], t[5], t[6], t[7])};
-}
-__device__ __noinline__ V8 sin8(V8 v) { return map8_unrolled(v, FSin()); }
-__device__ __noinline__ V8 cos8(V8 v) { return map8_unrolled(v, FCos()); }
-__device__ __noinline__ V8 exp8(V8 v) { return map8_unrolled(v, FExp()); }
-__device__ __noinline__ V8 log8(V8 v) { return map8_unrolled(v, FLog()); }
-__device__ __noinline__ V8 sqrt8(V8 v) { return map8_unrolled(v, FSqrt()); }
-// The EXT instantiation of the interpreter (programs that use 1/x, tan, asin,
-// acos, atan, tanh) runs twelve library routines: unrolled 8-wide they no
-// longer fit the instruction cache (ncu: 26 cycles per issue stalled on
-// instruction fetch, 23 % of issue slots used).  There the extended routines
-// run four cases at a time and the base ones two.  On a Table 1 population
-// (GPop/s, at 5 CTAs per SM): extended one at a time 1,600, two 1,708, four
-// 1,756, eight 1,383; base four at a time with extended four 1,309: the
-// instruction cache decides.  The base instantiation keeps its 8-wide copies
-// (4-wide: 2,662 -> 1,930 on base populations).
-template <typename F>
-__device__ __forceinline__ V8 map8_small(V8 v, F f) {
-  float t[8] = {v.a.x, v.a.y, v.a.z, v.a.w, v.b.x, v.b.y, v.b.z, v.b.w};
-#pragma unroll 4
-  for (int i = 0; i < 8; ++i) t[i] = f(t[i]);
-  return V8{make_float4(t[0], t[1], t[2], t[3]), make_float4(t[4], t[5], t[6], t[7])};
-}
-template <typename F>
-__device__ __forceinline__ V8 map8_base_small(V8 v, F f) {  // 2 in flight
-  float t[8] = {v.a.x, v.a.y, v.a.z, v.a.w, v.b.x, v.b.y, v.b.z, v.b.w};
-#pragma unroll 2
-  for (int i = 0; i < 8; ++i) t[i] = f(t[i]);
-  return V8{make_float4(t[0], t[1], t[2], t[3]), make_float4(t[4], t[5], t[6], t[7])};
-}
-__device__ __noinline__ V8 sin8s(V8 v) { return map8_base_small(v, FSin()); }
-__device__ __noinline__ V8 cos8s(V8 v) { return map8_base_small(v, FCos()); }
-__device__ __noinline__ V8 exp8s(V8 v) { return map8_base_small(v, FExp()); }
-__device__ __noinline__ V8 log8s(V8 v) { return map8_base_small(v, FLog()); }
-__device__ __noinline__ V8 sqrt8s(V8 v) { return map8_base_small(v, FSqrt()); }
-__device__ __noinline__ V8 div8s(V8 a, V8 b) {
-  float x[8] = {a.a.x, a.a.y, a.a.z, a.a.w, a.b.x, a.b.y, a.b.z, a.b.w};
-  const float y[8] = {b.a.x, b.a.y, b.a.z, b.a.w, b.b.x, b.b.y, b.b.z, b.b.w};
-#pragma unroll 2
-  for (int i = 0; i < 8; ++i) x[i] = op_div(x[i], y[i]);
-  return V8{make_float4(x[0], x[1], x[2], x[3]), make_float4(x[4], x[5], x[6], x[7])};
-}
-__device__ __noinline__ V8 ext8(uint32_t op, V8 v) {
-  switch (op) {
-    case OP_INV: return map8_small(v, FInv());
-    case OP_TAN: return map8_small(v, FTan());
-    case OP_ASIN: return map8_small(v, FAsin());
-    case OP_ACOS: return map8_small(v, FAcos());
-    case OP_ATAN: return map8_small(v, FAtan());
-    default: return map8_small(v, FTanh());
-  }
-}
-__device__ __noinline__ V8 div8(V8 a, V8 b) {
-  float x[8] = {a.a.x, a.a.y, a.a.z, a.a.w, a.b.x, a.b.y, a.b.z, a.b.w};
-  const float y[8] = {b.a.x, b.a.y, b.a.z, b.a.w, b.b.x, b.b.y, b.b.z, b.b.w};
-#pragma unroll MATH_UNROLL
-  for (int i = 0; i < 8; ++i) x[i] = op_div(x[i], y[i]);
-  return V8{make_float4(x[0], x[1], x[2], x[3]), make_float4(x[4], x[5], x[6], x[7])};
-}
-#define SIN8(v) sin8(v)
-#define COS8(v) cos8(v)
-#define EXP8(v) exp8(v)
-#define LOG8(v) log8(v)
-#define SQRT8(v) sqrt8(v)
-#define DIV8(p, q) div8(p, q)
-#define EXT8(op, v) ext8(op, v)
-
-// Runs the decoded program for this lane's 8 cases.  xa / xb point at the
-// lane's first and second case group in row 0 of X; `stk` at this lane's
-// entry of stack slot 0 in shared memory.
-// EXT: the copy of the loop that also runs 1/x, tan, asin, acos, atan, tanh
-template <bool EXT>
-__device__ __forceinline__ V8 interpret(const uint2 *__restrict__ code, int n, char *stk,
-                                        const float *__restrict__ xa, const float *__restrict__ xb) {
-  V8 T = splat8(0.f);
-  for (int ip = 0; ip < n; ++ip) {
-    const uint2 w = code[ip];
-    const uint32_t off = ins_off(w);
-    switch (ins_op(w)) {
-      case OP_LDV: T = ldX8(xa, xb, w.y); break;
-      case OP_LDC: T = splat8(__uint_as_float(w.y)); break;
-      case OP_PUSHV: st8(stk, off, T); T = ldX8(xa, xb, w.y); break;
-      case OP_PUSHC: st8(stk, off, T); T = splat8(__uint_as_float(w.y)); break;
-      case OP_ADD: { const V8 a = ld8(stk, off); T = ZIP8(f_add, a, T); } break;
-      case OP_SUB: { const V8 a = ld8(stk, off); T = ZIP8(f_sub, a, T); } break;
-      case OP_MUL: { const V8 a = ld8(stk, off); T = ZIP8(f_mul, a, T); } break;
-      case OP_DIV: { const V8 a = ld8(stk, off); T = EXT ? div8s(a, T) : DIV8(a, T); } break;
-      case OP_RSUB: { const V8 b = ld8(stk, off); T = ZIP8(f_sub, T, b); } break;
-      case OP_RDIV: { const V8 b = ld8(stk, off); T = EXT ? div8s(T, b) : DIV8(T, b); } break;
-      case OP_SIN: T = EXT ? sin8s(T) : SIN8(T); break;
-      case OP_COS: T = EXT ? cos8s(T) : COS8(T); break;
-      case OP_EXP: T = EXT ? exp8s(T) : EXP8(T); break;
-      case OP_LOG: T = EXT ? log8s(T) : LOG8(T); break;
-      case OP_SQRT: T = EXT ? sqrt8s(T) : SQRT8(T); break;
-      case OP_SQ: T = MAP8(f_sq, T); break;
-      case OP_INV:
-      case OP_TAN:
-      case OP_ASIN:
-      case OP_ACOS:
-      case OP_ATAN:
-      case OP_TANH:
-        if (EXT) T = EXT8(ins_op(w), T);
-        break;
-      case OP_VADD: { const V8 v = ldX8(xa, xb, w.y); T = ZIP8(f_add, T, v); } break;
-      case OP_VSUB: { const V8 v = ldX8(xa, xb, w.y); T = ZIP8(f_sub, T, v); } break;
-      case OP_VMUL: { const V8 v = ldX8(xa, xb, w.y); T = ZIP8(f_mul, T, v); } break;
-      case OP_VDIV: { const V8 v = ldX8(xa, xb, w.y); T = EXT ? div8s(T, v) : DIV8(T, v); } break;
-      case OP_VRSUB: { const V8 v = ldX8(xa, xb, w.y); T = ZIP8(f_sub, v, T); } break;
-      case OP_VRDIV: { const V8 v = ldX8(xa, xb, w.y); T = EXT ? div8s(v, T) : DIV8(v, T); } break;
-      case OP_CADD: { const V8 v = splat8(__uint_as_float(w.y)); T = ZIP8(f_add, T, v); } break;
-      case OP_CSUB: { const V8 v = splat8(__uint_as_float(w.y)); T = ZIP8(f_sub, T, v); } break;
-      case OP_CMUL: { const V8 v = splat8(__uint_as_float(w.y)); T = ZIP8(f_mul, T, v); } break;
-      case OP_CDIV: { const V8 v = splat8(__uint_as_float(w.y)); T = EXT ? div8s(T, v) : DIV8(T, v); } break;
-      case OP_CRSUB: { const V8 v = splat8(__uint_as_float(w.y)); T = ZIP8(f_sub, v, T); } break;
-      case OP_CRDIV: { const V8 v = splat8(__uint_as_float(w.y)); T = EXT ? div8s(v, T) : DIV8(v, T); } break;
-      default: break;
-    }
-  }
-  return T;
 }
 
 // ---------------------------------------------------------------- reductions
@@ -449,7 +295,8 @@ __device__ __forceinline__ int p2p_case(float yh, float y, int M, float Mf, floa
 // Out of line: the copy inside the interpreter loop measured 1.7 % slower.
 struct R4Part { float s1, s2, s3, s4, s5; int n1, n2; };
 __device__ __noinline__ R4Part r4_part(V8 T, float4 ya, float4 yb, int nvalid, float shift) {
-  const float tv[CPL] = {T.a.x, T.a.y, T.a.z, T.a.w, T.b.x, T.b.y, T.b.z, T.b.w};
+  float tv[CPL];
+  unpack8(T, tv);
   const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
   float d[CPL], e[CPL];
   int c1 = 0, c2 = 0;
@@ -491,10 +338,98 @@ __device__ __forceinline__ WarpSmem warp_smem(unsigned char *smem, int warp, int
   return w;
 }
 
+// A lane's running sums over an item's cases.
+struct Acc {
+  Kahan se, s1, s2, s3, s4, s5;
+  float shift;
+  int c1, c2;
+  long long score;
+};
+
+// Adds one step's 8 outputs per lane (cases c0 .. c0 + 7, those below cend
+// valid; cl / cl4 the readable positions of the two halves of the target) to
+// the sums of the mode.  MODE_BOTH takes those selected by `want` (bit 0:
+// squared error, bit 1: correlation moments).  y: the target (MSE, Eq. 3) with
+// N values; yc: the centred target (1 - r^2, Eq. 2).
+template <int MODE>
+__device__ __noinline__ void accumulate(Acc *acc, V8 T, int c0, int cl, int cl4, int cend, int first,
+                                  const float *__restrict__ y, const float *__restrict__ yc, int N, int want, int M) {
+  const bool do_mse = MODE == MODE_MSE || (MODE == MODE_BOTH && (want & 1));
+  const bool do_corr = MODE == MODE_CORR || (MODE == MODE_BOTH && (want & 2));
+  float tv[CPL];
+  unpack8(T, tv);
+  bool ok[CPL];
+#pragma unroll
+  for (int i = 0; i < CPL; ++i) ok[i] = c0 + i < cend;
+  if (do_mse) {
+    const float4 ya = load_y4(y, cl, N), yb = load_y4(y, cl4, N);
+    const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+    float e[CPL];
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) e[i] = sel(ok[i], tv[i] - yv[i]);
+    acc->se.add(((e[0] * e[0] + e[1] * e[1]) + (e[2] * e[2] + e[3] * e[3])) +
+                ((e[4] * e[4] + e[5] * e[5]) + (e[6] * e[6] + e[7] * e[7])));
+  }
+  if (do_corr) {
+    if (first) acc->shift = __shfl_sync(FULL, tv[0], 0);
+    const float shift = acc->shift;
+    const float4 ya = ldx4(yc + cl), yb = ldx4(yc + cl4);
+    const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+    float d[CPL];
+#pragma unroll
+    for (int i = 0; i < CPL; ++i) d[i] = sel(ok[i], tv[i] - shift);
+    acc->s1.add(((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])));
+    acc->s2.add(((d[0] * d[0] + d[1] * d[1]) + (d[2] * d[2] + d[3] * d[3])) +
+                ((d[4] * d[4] + d[5] * d[5]) + (d[6] * d[6] + d[7] * d[7])));
+    acc->s3.add(((d[0] * yv[0] + d[1] * yv[1]) + (d[2] * yv[2] + d[3] * yv[3])) +
+                ((d[4] * yv[4] + d[5] * yv[5]) + (d[6] * yv[6] + d[7] * yv[7])));
+  }
+  if (MODE == MODE_R4) {
+    // pairs: both finite -> moments; one invalid -> c1; both -> c2.  yc
+    // holds y - ybar for finite y and NaN for invalid targets.
+    if (first) {
+      const unsigned fin = __ballot_sync(FULL, isfinite(tv[0]));
+      acc->shift = fin ? __shfl_sync(FULL, tv[0], __ffs(fin) - 1) : 0.0f;
+    }
+    const float4 ya = ldx4(yc + cl), yb = ldx4(yc + cl4);
+    const R4Part q = r4_part(T, ya, yb, cend - c0, acc->shift);
+    acc->s1.add(q.s1);
+    acc->s2.add(q.s2);
+    acc->s3.add(q.s3);
+    acc->s4.add(q.s4);
+    acc->s5.add(q.s5);
+    acc->c1 += q.n1;
+    acc->c2 += q.n2;
+  }
+  if (MODE == MODE_P2P) {
+    const float Mf = (float)M, pen = __fdiv_rn(Mf, 11.0f);
+    const float4 ya = load_y4(y, cl, N), yb = load_y4(y, cl4, N);
+    // one copy of the per-case body: the values rotate through it
+    float t0 = tv[0], t1 = tv[1], t2 = tv[2], t3 = tv[3], t4 = tv[4], t5 = tv[5], t6 = tv[6], t7 = tv[7];
+    float y0 = ya.x, y1 = ya.y, y2 = ya.z, y3 = ya.w, y4 = yb.x, y5 = yb.y, y6 = yb.z, y7 = yb.w;
+    int c1 = 0, c2 = 0;
+    long long score = 0;
+#pragma unroll 1
+    for (int i = 0; i < CPL; ++i) {
+      if (c0 + i < cend) {
+        const bool vh = isfinite(t0), vy = isfinite(y0);
+        c1 += vh != vy ? 1 : 0;
+        c2 += (!vh && !vy) ? 1 : 0;
+        score += p2p_case(t0, y0, M, Mf, pen);
+      }
+      t0 = t1; t1 = t2; t2 = t3; t3 = t4; t4 = t5; t5 = t6; t6 = t7;
+      y0 = y1; y1 = y2; y2 = y3; y3 = y4; y4 = y5; y5 = y6; y6 = y7;
+    }
+    acc->c1 += c1;
+    acc->c2 += c2;
+    acc->score += score;
+  }
+}
+
 // Evaluates program `prog` of problem p on case chunk `c` with the calling
 // warp.  MODE_BOTH accumulates the sums selected by `want` (bit 0: squared
 // error, bit 1: correlation moments); the other modes ignore `want`.
-template <int MODE, bool EXT>
+template <int MODE, bool EXT, bool WIDE>
 __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, const WarpSmem &w,
                                           int lane, int want) {
   const bool do_mse = MODE == MODE_MSE || (MODE == MODE_BOTH && (want & 1));
@@ -512,100 +447,45 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
   __syncwarp();  // the previous item is done reading the code
   const uint2 *src = p.code + (size_t)prog * p.Lmax;
   for (int i = lane; i < n; i += 32) w.code[i] = src[i];
+  if (lane == 0) w.code[n] = make_uint2(OP_END, 0u);
   __syncwarp();
 
   char *stk = w.stk + lane * 16;
   const int last_group = (cend - 1) & ~(CPL - 1);
 
-  Kahan se, s1, s2, s3, s4, s5;
-  float shift = 0.f;
-  long long score = 0;
-  int c1 = 0, c2 = 0;
-  const float Mf = (float)p.score_M, pen = __fdiv_rn(Mf, 11.0f);
+  Acc acc;
+  acc.se = acc.s1 = acc.s2 = acc.s3 = acc.s4 = acc.s5 = Kahan();
+  acc.shift = 0.f;
+  acc.c1 = acc.c2 = 0;
+  acc.score = 0;
   for (int base = cbeg; base < cend; base += STEP) {
     const int c0 = base + CPL * lane;
     const int cl = c0 < cend ? c0 : last_group;           // first 4 cases, always readable
     const int cl4 = cl + 4 < cend ? cl + 4 : cl;          // second 4, or a re-read when none valid
-    const V8 T = interpret<EXT>(w.code, n, stk, p.X + cl, p.X + cl4);
-    const float tv[CPL] = {T.a.x, T.a.y, T.a.z, T.a.w, T.b.x, T.b.y, T.b.z, T.b.w};
-    bool ok[CPL];
-#pragma unroll
-    for (int i = 0; i < CPL; ++i) ok[i] = c0 + i < cend;
+    const V8 T = interpret<EXT, WIDE, MODE == MODE_P2P>(w.code, stk, p.X + cl, p.X + cl4);
     if (MODE == MODE_PREDICT) {
+      float tv[CPL];
+      unpack8(T, tv);
       float *row = p.yhat + (size_t)prog * p.ldy;
 #pragma unroll
       for (int i = 0; i < CPL; ++i)
-        if (ok[i]) row[c0 + i] = tv[i];
-    }
-    if (do_mse) {
-      const float4 ya = load_y4(p.y, cl, p.N), yb = load_y4(p.y, cl4, p.N);
-      const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-      float e[CPL];
-#pragma unroll
-      for (int i = 0; i < CPL; ++i) e[i] = sel(ok[i], tv[i] - yv[i]);
-      se.add(((e[0] * e[0] + e[1] * e[1]) + (e[2] * e[2] + e[3] * e[3])) +
-             ((e[4] * e[4] + e[5] * e[5]) + (e[6] * e[6] + e[7] * e[7])));
-    }
-    if (do_corr) {
-      if (base == cbeg) shift = __shfl_sync(FULL, T.a.x, 0);
-      const float4 ya = ldx4(p.yc + cl), yb = ldx4(p.yc + cl4);
-      const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-      float d[CPL];
-#pragma unroll
-      for (int i = 0; i < CPL; ++i) d[i] = sel(ok[i], tv[i] - shift);
-      s1.add(((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7])));
-      s2.add(((d[0] * d[0] + d[1] * d[1]) + (d[2] * d[2] + d[3] * d[3])) +
-             ((d[4] * d[4] + d[5] * d[5]) + (d[6] * d[6] + d[7] * d[7])));
-      s3.add(((d[0] * yv[0] + d[1] * yv[1]) + (d[2] * yv[2] + d[3] * yv[3])) +
-             ((d[4] * yv[4] + d[5] * yv[5]) + (d[6] * yv[6] + d[7] * yv[7])));
-    }
-    if (MODE == MODE_R4) {
-      // pairs: both finite -> moments; one invalid -> c1; both -> c2.  yc
-      // holds y - ybar for finite y and NaN for invalid targets.
-      if (base == cbeg) {
-        const unsigned fin = __ballot_sync(FULL, isfinite(T.a.x));
-        shift = fin ? __shfl_sync(FULL, T.a.x, __ffs(fin) - 1) : 0.0f;
-      }
-      const float4 ya = ldx4(p.yc + cl), yb = ldx4(p.yc + cl4);
-      const R4Part q = r4_part(T, ya, yb, cend - c0, shift);
-      s1.add(q.s1);
-      s2.add(q.s2);
-      s3.add(q.s3);
-      s4.add(q.s4);
-      s5.add(q.s5);
-      c1 += q.n1;
-      c2 += q.n2;
-    }
-    if (MODE == MODE_P2P) {
-      const float4 ya = load_y4(p.y, cl, p.N), yb = load_y4(p.y, cl4, p.N);
-      // one copy of the per-case body: the values rotate through it
-      float t0 = T.a.x, t1 = T.a.y, t2 = T.a.z, t3 = T.a.w, t4 = T.b.x, t5 = T.b.y, t6 = T.b.z, t7 = T.b.w;
-      float y0 = ya.x, y1 = ya.y, y2 = ya.z, y3 = ya.w, y4 = yb.x, y5 = yb.y, y6 = yb.z, y7 = yb.w;
-#pragma unroll 1
-      for (int i = 0; i < CPL; ++i) {
-        if (c0 + i < cend) {
-          const bool vh = isfinite(t0), vy = isfinite(y0);
-          c1 += vh != vy ? 1 : 0;
-          c2 += (!vh && !vy) ? 1 : 0;
-          score += p2p_case(t0, y0, p.score_M, Mf, pen);
-        }
-        t0 = t1; t1 = t2; t2 = t3; t3 = t4; t4 = t5; t5 = t6; t6 = t7;
-        y0 = y1; y1 = y2; y2 = y3; y3 = y4; y4 = y5; y5 = y6; y6 = y7;
-      }
+        if (c0 + i < cend) row[c0 + i] = tv[i];
+    } else {
+      accumulate<MODE>(&acc, T, c0, cl, cl4, cend, base == cbeg, p.y, p.yc, p.N, want, p.score_M);
     }
   }
   if (MODE != MODE_PREDICT) {
     double *rec = p.partials + ((size_t)prog * p.nchunks + c) * PSTRIDE;
     if (do_mse) {
-      const double v = warp_sum(se.value());
+      const double v = warp_sum(acc.se.value());
       if (lane == 0) rec[0] = v;
     }
     if (do_corr) {
-      const double a = warp_sum(s1.value());
-      const double b = warp_sum(s2.value());
-      const double d = warp_sum(s3.value());
+      const double a = warp_sum(acc.s1.value());
+      const double b = warp_sum(acc.s2.value());
+      const double d = warp_sum(acc.s3.value());
       if (lane == 0) {
-        rec[1] = (double)shift;
+        rec[1] = (double)acc.shift;
         rec[2] = a;
         rec[3] = b;
         rec[4] = d;
@@ -613,11 +493,11 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
     }
     if (MODE == MODE_R4) {
       // [shift, sum d, sum d^2, sum d e, sum e, sum e^2, c1, c2]
-      const double v1 = warp_sum(s1.value()), v2 = warp_sum(s2.value()), v3 = warp_sum(s3.value());
-      const double v4 = warp_sum(s4.value()), v5 = warp_sum(s5.value());
-      const double n1 = warp_sum((double)c1), n2 = warp_sum((double)c2);
+      const double v1 = warp_sum(acc.s1.value()), v2 = warp_sum(acc.s2.value()), v3 = warp_sum(acc.s3.value());
+      const double v4 = warp_sum(acc.s4.value()), v5 = warp_sum(acc.s5.value());
+      const double n1 = warp_sum((double)acc.c1), n2 = warp_sum((double)acc.c2);
       if (lane == 0) {
-        rec[0] = (double)shift;
+        rec[0] = (double)acc.shift;
         rec[1] = v1;
         rec[2] = v2;
         rec[3] = v3;
@@ -629,8 +509,8 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
     }
     if (MODE == MODE_P2P) {
       // [sum of the integer scores (exact), c1, c2]
-      const double v = warp_sum((double)score);
-      const double n1 = warp_sum((double)c1), n2 = warp_sum((double)c2);
+      const double v = warp_sum((double)acc.score);
+      const double n1 = warp_sum((double)acc.c1), n2 = warp_sum((double)acc.c2);
       if (lane == 0) {
         rec[0] = v;
         rec[6] = n1;
@@ -641,30 +521,43 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
 }
 
 // ---------------------------------------------------------------- single problem
-// Up to three passes over the work items: EXT = false takes the programs of
-// the base operators (and the invalid ones), EXT = true those that use 1/x,
-// tan, asin, acos, atan or tanh; it returns at once when the decoder counted
-// none.  Keeping the extended operators out of the first kernel keeps its
-// loop (and its speed) what it is for the base operators.  Both give each
-// warp shallow_slots(Lmax, MINB) stack slots; the programs that need more
-// (NCODE_DEEP) run in a third launch of the EXT kernel with deep = 1 and
-// slots_for(Lmax) slots, made only when the two differ.
-template <int MODE, bool EXT, int MINB>
+// Up to three passes over the work items: the programs of the base operators
+// (and the invalid ones), those that use 1/x, tan, asin, acos, atan or tanh
+// (which returns at once when the decoder counted none), and those that need
+// more than the main passes' shallow_slots(Lmax, MINB) stack slots (NCODE_DEEP;
+// made only when slots_for(Lmax) is more).  Keeping the extended operators out
+// of the first kernel keeps its loop inside the instruction cache.  Where the
+// rows of X could not be laid out for 256-bit loads, one pass of the EXT kernel
+// without them takes the base and the extended programs.
+enum Pass { PASS_BASE = 0, PASS_EXT = 1, PASS_DEEP = 2, PASS_SHALLOW = 3 };
+
+__device__ __forceinline__ bool takes(int pass, int ncode) {
+  if (pass == PASS_DEEP) return ncode_deep(ncode);
+  if (ncode_deep(ncode)) return false;
+  return pass == PASS_SHALLOW || ncode_ext(ncode) == (pass == PASS_EXT);
+}
+// the pass's work counter; NULL when it has no programs
+__device__ __forceinline__ unsigned long long *pass_queue(unsigned long long *queue, int pass) {
+  if (pass == PASS_EXT) return queue[2] ? queue + 1 : nullptr;
+  if (pass == PASS_DEEP) return queue[4] ? queue + 3 : nullptr;
+  return queue;
+}
+
+template <int MODE, bool EXT, bool WIDE, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB) eval_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const bool deep = EXT && p.deep;  // the deep pass runs the EXT copy of the loop
-  if (deep ? p.queue[4] == 0 : (EXT && p.queue[2] == 0)) return;
+  const int pass = EXT ? p.pass : PASS_BASE;
+  unsigned long long *q = pass_queue(p.queue, pass);
+  if (!q) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, p.warp_bytes, p.slots);
-  unsigned long long *q = p.queue + (deep ? 3 : (EXT ? 1 : 0));
   for (;;) {
     const long long item = next_item(q, p.total_items, p.abort, p.err, lane);
     if (item >= p.total_items) break;
     const int c = (int)(item / (unsigned long long)p.P);
     const int prog = (int)(item % (unsigned long long)p.P);
-    const int nc = p.ncode[prog];
-    if (deep ? !ncode_deep(nc) : (nc & (NCODE_EXT | NCODE_DEEP)) != (EXT ? NCODE_EXT : 0)) continue;
-    eval_item<MODE, EXT>(p, c, prog, w, lane, 3);
+    if (!takes(pass, p.ncode[prog])) continue;
+    eval_item<MODE, EXT, WIDE>(p, c, prog, w, lane, 3);
   }
 }
 
@@ -693,6 +586,9 @@ struct BatchProblem {
   int corr_chunk_begin;  // first block of this problem in the batched centring launch (-1: none)
   int xform;             // >= 1: X / ldx are the problem's variable table of this depth (EvalParams::xform)
   uint8_t *xneed;
+  const float *Xsrc;     // as EvalParams::Xsrc
+  long long ldsrc;
+  int stage_begin;       // first staging block of this problem in the decode launch
 };
 
 struct BatchParams {
@@ -706,7 +602,8 @@ struct BatchParams {
   int warp_bytes;
   int slots;
   int maxL;                   // the largest Lmax of the batch
-  int deep;                   // as EvalParams::deep
+  int pass;                   // as EvalParams::pass
+  int decode_blocks, stage_blocks;  // blocks of the decode launch that decode, then those that copy X
   const int32_t *abort;       // as EvalParams::abort
   unsigned *err;
 };
@@ -735,6 +632,8 @@ __device__ __forceinline__ EvalParams view(const BatchProblem &q) {
   p.ncode = q.ncode;
   p.xform = q.xform;
   p.xneed = q.xneed;
+  p.Xsrc = q.Xsrc;
+  p.ldsrc = q.ldsrc;
   return p;
 }
 
@@ -742,6 +641,14 @@ __device__ __forceinline__ EvalParams view(const BatchProblem &q) {
 // for the batch's largest Lmax, b.maxL)
 __global__ void decode_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  if ((int)blockIdx.x >= b.decode_blocks) {
+    const int r = (int)blockIdx.x - b.decode_blocks;
+    int i = 0;
+    while (i + 1 < b.nprob && b.prob[i + 1].stage_begin <= r) ++i;
+    const EvalParams p = view(b.prob[i]);
+    if (p.Xsrc) stage_rows(p, r - b.prob[i].stage_begin);
+    return;
+  }
   const int warp = threadIdx.x >> 5;
   const int g = blockIdx.x * (blockDim.x >> 5) + warp;
   if (g >= b.total_progs) return;
@@ -759,18 +666,17 @@ __global__ void decode_batched_kernel(const __grid_constant__ BatchParams b) {
 
 // Work items of every problem come from one atomic counter: problem q owns
 // items [item_begin_q, item_begin_q + P_q * nchunks_q), chunk-major inside.
-// EXT and deep as for eval_kernel (the extended programs of every problem
-// in a second launch, the deep ones in a third).
+// Passes as for eval_kernel.
 // At most 64 registers, so that 4 CTAs fit an SM (75 unbounded, 3 CTAs):
-// 2,608 -> 2,949 GPop/s on the 64-problem batch despite a few spilled values.
-template <bool EXT, int MINB>
+// 2,608 -> 2,949 GPop/s on the 64-problem batch.
+template <bool EXT, bool WIDE, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const bool deep = EXT && b.deep;
-  if (deep ? b.queue[4] == 0 : (EXT && b.queue[2] == 0)) return;
+  const int pass = EXT ? b.pass : PASS_BASE;
+  unsigned long long *qc = pass_queue(b.queue, pass);
+  if (!qc) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, b.warp_bytes, b.slots);
-  unsigned long long *qc = b.queue + (deep ? 3 : (EXT ? 1 : 0));
   for (;;) {
     const long long item = next_item(qc, b.total_items, b.abort, b.err, lane);
     if (item >= b.total_items) break;
@@ -785,10 +691,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __
     const long long local = (long long)item - q.item_begin;
     const int c = (int)(local / q.P);
     const int prog = (int)(local % q.P);
-    const int nc = q.ncode[prog];
-    if (deep ? !ncode_deep(nc) : (nc & (NCODE_EXT | NCODE_DEEP)) != (EXT ? NCODE_EXT : 0)) continue;
+    if (!takes(pass, q.ncode[prog])) continue;
     const int want = q.mode == MODE_MSE ? 1 : (q.mode == MODE_CORR ? 2 : 3);
-    eval_item<MODE_BOTH, EXT>(p, c, prog, w, lane, want);
+    eval_item<MODE_BOTH, EXT, WIDE>(p, c, prog, w, lane, want);
   }
 }
 
@@ -1083,59 +988,57 @@ __global__ void finalize_batched_kernel(const __grid_constant__ BatchParams b) {
 }
 
 // ---------------------------------------------------------------- host side
-template <int MODE, bool EXT, int MINB>
-sr_status occupancy_grid(sr_ctx *ctx, int smem, int *grid) {
-  sr_status st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(eval_kernel<MODE, EXT, MINB>));
+typedef void (*EvalKernel)(EvalParams);
+
+// The instantiations: base and EXT with 4 or 5 CTAs per SM, and the EXT one
+// that reads rows in halves (4 CTAs).
+template <int MODE>
+EvalKernel eval_kernel_m(bool ext, bool wide, int minb) {
+  if (!wide) return eval_kernel<MODE, true, false, 4>;
+  if (minb == 5) return ext ? eval_kernel<MODE, true, true, 5> : eval_kernel<MODE, false, true, 5>;
+  return ext ? eval_kernel<MODE, true, true, 4> : eval_kernel<MODE, false, true, 4>;
+}
+EvalKernel eval_kernel_for(int mode, bool ext, bool wide, int minb) {
+  switch (mode) {
+    case MODE_PREDICT: return eval_kernel_m<MODE_PREDICT>(ext, wide, minb);
+    case MODE_MSE: return eval_kernel_m<MODE_MSE>(ext, wide, minb);
+    case MODE_CORR: return eval_kernel_m<MODE_CORR>(ext, wide, minb);
+    case MODE_R4: return eval_kernel_m<MODE_R4>(ext, wide, minb);
+    case MODE_P2P: return eval_kernel_m<MODE_P2P>(ext, wide, minb);
+    default: return eval_kernel_m<MODE_BOTH>(ext, wide, minb);
+  }
+}
+
+// CTAs of `kernel` with `smem` bytes each on the whole GPU
+sr_status persistent_grid(sr_ctx *ctx, const void *kernel, int smem, int *grid) {
+  sr_status st = allow_dynamic_smem(ctx, kernel);
   if (st != SR_OK) return st;
   int nb = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_kernel<MODE, EXT, MINB>, WARPS * 32, smem);
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, WARPS * 32, smem);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
   if (nb < 1) return fail(ctx, SR_EINVAL, "Lmax too large for shared memory");
   *grid = nb * ctx->num_sms;
   return SR_OK;
 }
 
-template <bool EXT, int MINB>
-sr_status grid_for_m(sr_ctx *ctx, int mode, int smem, int *grid) {
-  switch (mode) {
-    case MODE_PREDICT: return occupancy_grid<MODE_PREDICT, EXT, MINB>(ctx, smem, grid);
-    case MODE_MSE: return occupancy_grid<MODE_MSE, EXT, MINB>(ctx, smem, grid);
-    case MODE_CORR: return occupancy_grid<MODE_CORR, EXT, MINB>(ctx, smem, grid);
-    case MODE_R4: return occupancy_grid<MODE_R4, EXT, MINB>(ctx, smem, grid);
-    case MODE_P2P: return occupancy_grid<MODE_P2P, EXT, MINB>(ctx, smem, grid);
-    default: return occupancy_grid<MODE_BOTH, EXT, MINB>(ctx, smem, grid);
-  }
-}
-
-template <bool EXT>
-sr_status grid_for_t(sr_ctx *ctx, int mode, int minb, int smem, int *grid) {
-  return minb == 5 ? grid_for_m<EXT, 5>(ctx, mode, smem, grid) : grid_for_m<EXT, 4>(ctx, mode, smem, grid);
-}
-
-template <bool EXT, int MINB>
-void launch_mode_m(int mode, int grid, int smem, cudaStream_t s, const EvalParams &ep) {
-  switch (mode) {
-    case MODE_PREDICT: eval_kernel<MODE_PREDICT, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-    case MODE_MSE: eval_kernel<MODE_MSE, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-    case MODE_CORR: eval_kernel<MODE_CORR, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-    case MODE_R4: eval_kernel<MODE_R4, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-    case MODE_P2P: eval_kernel<MODE_P2P, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-    default: eval_kernel<MODE_BOTH, EXT, MINB><<<grid, WARPS * 32, smem, s>>>(ep); break;
-  }
-}
-
-template <bool EXT>
-void launch_mode(int mode, int minb, int grid, int smem, cudaStream_t s, const EvalParams &ep) {
-  if (minb == 5) launch_mode_m<EXT, 5>(mode, grid, smem, s, ep);
-  else launch_mode_m<EXT, 4>(mode, grid, smem, s, ep);
+sr_status launch_pass(sr_ctx *ctx, int mode, bool ext, bool wide, int minb, int smem, const EvalParams &ep) {
+  const EvalKernel k = eval_kernel_for(mode, ext, wide, minb);
+  int grid = 0;
+  sr_status st = persistent_grid(ctx, reinterpret_cast<const void *>(k), smem, &grid);
+  if (st != SR_OK) return st;
+  k<<<grid, WARPS * 32, smem, ctx->stream>>>(ep);
+  ctx->launches += 1;
+  return SR_OK;
 }
 
 struct Plan {
   int minb;       // CTAs per SM of the main passes (eval_kernel's MINB)
   int slots;      // stack slots per warp of the main passes
-  int grid, smem, chunk, nchunks;
+  int smem, chunk, nchunks;
   int smem_deep;  // shared memory of the deep pass (0: none)
   long long items;
+  bool wide;      // the rows of X are laid out for 256-bit loads (its own, or the table's)
+  bool stage;     // X is copied to the table's first rows (no transforms)
   int xform;      // the variable table's depth (0: none; rows of ldxt floats)
   int ldxt;
   size_t off_queue, off_flags, off_ncode, off_code, off_part, off_yc,
@@ -1147,22 +1050,29 @@ struct Plan {
 // (0: no; 1: u(x_j); 2: also the compositions, where the table stays
 // within XFORM2_MAX_BYTES), and that table's row stride.
 inline int use_xform(const sr_ctx *ctx, int P, int nvars, int N, int *ldxt) {
-  *ldxt = (N + 3) / 4 * 4;
+  *ldxt = (int)align_up((size_t)N, CPL);  // whole groups of 8 cases (sr_vm.cuh, WIDE)
   const bool automatic = ctx->xform == 1 && N >= XFORM_MIN_N && P >= XFORM_MIN_P;
   if (!(ctx->xform == 2 || automatic)) return 0;
-  const long long cells2 = (long long)xform_rows(nvars, 2) * *ldxt;
+  const long long cells2 = (long long)xform_rows(nvars, 2) * align_up((size_t)N, 4);
   if (cells2 < 0xFFFFFFFFll && cells2 * 4 <= XFORM2_MAX_BYTES) return 2;
   return (long long)xform_rows(nvars, 1) * *ldxt < 0xFFFFFFFFll ? 1 : 0;
 }
 
-sr_status make_plan(sr_ctx *ctx, int mode, int P, int Lmax, int N, Plan *pl, int nvars = 1) {
+// whether rows of X at this address and stride can be read by 256-bit loads
+// (8 cases from any multiple of 8 on)
+inline bool rows_are_wide(const float *X, long long ldx) { return ((uintptr_t)X & 31) == 0 && ldx % CPL == 0; }
+
+// How a call lays out its rows: the variable table, a copy of X where X itself
+// is not laid out for wide loads, or X as it is.
+enum Layout { LAY_TABLE, LAY_COPY, LAY_PLAIN };
+
+void make_plan(sr_ctx *ctx, int P, int Lmax, int N, Plan *pl, int nvars, bool x_wide, Layout lay) {
   pl->minb = eval_minb(Lmax, ctx->eval_ctas);
   pl->slots = shallow_slots(Lmax, pl->minb);
   pl->smem = WARPS * warp_smem_bytes(pl->slots, Lmax);
   pl->smem_deep = slots_for(Lmax) > pl->slots ? WARPS * warp_smem_bytes(slots_for(Lmax), Lmax) : 0;
-  sr_status st = grid_for_t<false>(ctx, mode, pl->minb, pl->smem, &pl->grid);
-  if (st != SR_OK) return st;
-  const long long warps = (long long)pl->grid * WARPS;
+  const long long warps =
+      (long long)chunk_ctas(Lmax, chunk_minb(Lmax, ctx->eval_ctas)) * ctx->num_sms * WARPS;
   const long long want = warps * TARGET_ITEMS_PER_WARP;
   int nch = (int)((want + P - 1) / (P > 0 ? P : 1));
   // chunks of at least one warp step: a small problem (few programs, few
@@ -1171,6 +1081,9 @@ sr_status make_plan(sr_ctx *ctx, int mode, int P, int Lmax, int N, Plan *pl, int
   nch = nch < 1 ? 1 : (nch > max_chunks ? max_chunks : nch);
   int chunk = (N + nch - 1) / nch;
   pl->xform = use_xform(ctx, P, nvars, N, &pl->ldxt);
+  if (lay != LAY_TABLE) pl->xform = 0;
+  pl->stage = !pl->xform && !x_wide && lay != LAY_PLAIN;
+  pl->wide = pl->xform || pl->stage || x_wide;
   if (ctx->tile_cases > 0) {
     chunk = ctx->tile_cases;  // autotuned cases per work item
   } else if (pl->xform) {
@@ -1199,9 +1112,10 @@ sr_status make_plan(sr_ctx *ctx, int mode, int P, int Lmax, int N, Plan *pl, int
     const size_t rows = (size_t)xform_rows(nvars, pl->xform);
     pl->off_xt = cv.take(rows * pl->ldxt * 4);
     pl->off_xneed = cv.take(rows - nvars);
+  } else if (pl->stage) {
+    pl->off_xt = cv.take((size_t)nvars * pl->ldxt * 4);
   }
   pl->bytes = cv.off;
-  return SR_OK;
 }
 
 sr_status check_common(sr_ctx *ctx, const uint8_t *programs, const int32_t *lengths,
@@ -1232,15 +1146,14 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
                       int ldy, int M = 0, int32_t *counts = nullptr) {
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
   Plan pl;
-  sr_status st = make_plan(ctx, mode, P, Lmax, N, &pl, nvars);
-  if (st != SR_OK) return st;
-  st = ensure_workspace(ctx, pl.bytes);
-  if (st == SR_ENOMEM && pl.xform) {  // no room for the variable table: evaluate without it
-    const int mode_x = ctx->xform;
-    ctx->xform = 0;
-    st = make_plan(ctx, mode, P, Lmax, N, &pl, nvars);
-    ctx->xform = mode_x;
-    if (st == SR_OK) st = ensure_workspace(ctx, pl.bytes);
+  const bool x_wide = rows_are_wide(X, ldx);
+  // with less room (as inside stream capture): without the variable table,
+  // then without a copy of X
+  sr_status st = SR_ENOMEM;
+  for (Layout lay : {LAY_TABLE, LAY_COPY, LAY_PLAIN}) {
+    make_plan(ctx, P, Lmax, N, &pl, nvars, x_wide, lay);
+    st = ensure_workspace(ctx, pl.bytes);
+    if (st != SR_ENOMEM) break;
   }
   if (st != SR_OK) return st;
   char *ws = ctx->ws;
@@ -1271,31 +1184,29 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   ep.ldy = ldy;
   ep.slots = pl.slots;
   ep.warp_bytes = warp_smem_bytes(pl.slots, Lmax);
-  ep.deep = 0;
+  ep.pass = PASS_BASE;
   ep.abort = ctx->abort_flag;
   ep.err = ctx->dev_words;
   ep.score_M = M;
   ep.xform = pl.xform;
   ep.xneed = pl.xform ? reinterpret_cast<uint8_t *>(ws + pl.off_xneed) : nullptr;
-  if (pl.xform) {  // the kernels read the variable table; the decoder writes its row offsets
+  if (pl.xform || pl.stage) {  // the kernels read the table's rows; the decoder writes its row offsets
     ep.X = reinterpret_cast<const float *>(ws + pl.off_xt);
     ep.ldx = pl.ldxt;
   }
-
-  int grid_ext = 0, grid_deep = 0;
-  st = grid_for_t<true>(ctx, mode, pl.minb, pl.smem, &grid_ext);
-  if (st != SR_OK) return st;
-  if (pl.smem_deep) {
-    st = grid_for_t<true>(ctx, mode, 4, pl.smem_deep, &grid_deep);
-    if (st != SR_OK) return st;
+  if (pl.stage) {
+    ep.Xsrc = X;
+    ep.ldsrc = ldx;
   }
+
   SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.queue, 0, 5 * sizeof(unsigned long long), s));
   if (pl.xform) SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.xneed, 0, (size_t)(xform_rows(nvars, pl.xform) - nvars), s));
   // one warp per block spreads the serial per-program decode over the SMs
   st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(decode_kernel));
   if (st != SR_OK) return st;
-  decode_kernel<<<(P + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32, DECODE_WARPS * decode_warp_bytes(Lmax),
-                  s>>>(ep);
+  const int stage = pl.stage ? stage_blocks(nvars, N) : 0;
+  decode_kernel<<<(P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
+                  DECODE_WARPS * decode_warp_bytes(Lmax), s>>>(ep);
   ctx->launches += 1;
   if (pl.xform) {
     const dim3 g((unsigned)((N + XF_THREADS * 4 - 1) / (XF_THREADS * 4)), (unsigned)xform_rows(nvars, pl.xform));
@@ -1312,17 +1223,21 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
                                                       const_cast<float *>(ep.yc), ych);
     ctx->launches += 2;
   }
-  launch_mode<false>(mode, pl.minb, pl.grid, pl.smem, s, ep);
-  launch_mode<true>(mode, pl.minb, grid_ext, pl.smem, s, ep);
-  ctx->launches += 2;
-  if (pl.smem_deep) {
-    EvalParams ed = ep;
-    ed.deep = 1;
-    ed.slots = slots_for(Lmax);
-    ed.warp_bytes = warp_smem_bytes(ed.slots, Lmax);
-    launch_mode<true>(mode, 4, grid_deep, pl.smem_deep, s, ed);
-    ctx->launches += 1;
+  if (pl.wide) {
+    st = launch_pass(ctx, mode, false, true, pl.minb, pl.smem, ep);
+    ep.pass = PASS_EXT;
+    if (st == SR_OK) st = launch_pass(ctx, mode, true, true, pl.minb, pl.smem, ep);
+  } else {
+    ep.pass = PASS_SHALLOW;
+    st = launch_pass(ctx, mode, true, false, 4, pl.smem, ep);
   }
+  if (st == SR_OK && pl.smem_deep) {
+    ep.pass = PASS_DEEP;
+    ep.slots = slots_for(Lmax);
+    ep.warp_bytes = warp_smem_bytes(ep.slots, Lmax);
+    st = launch_pass(ctx, mode, true, pl.wide, 4, pl.smem_deep, ep);
+  }
+  if (st != SR_OK) return st;
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   if (mode != MODE_PREDICT) {
     FinalParams fp{ep.partials, ep.flags, ych, P, N, pl.chunk, pl.nchunks, mode, fitness, M, counts};
@@ -1334,29 +1249,21 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
 }
 
 // ---------------------------------------------------------------- batched host side
-template <bool EXT, int MINB>
-sr_status batched_grid_m(sr_ctx *ctx, int smem, int *grid) {
-  sr_status st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(eval_batched_kernel<EXT, MINB>));
+typedef void (*BatchKernel)(const BatchParams);
+BatchKernel batch_kernel_for(bool ext, bool wide, int minb) {
+  if (!wide) return eval_batched_kernel<true, false, 4>;
+  if (minb == 3) return ext ? eval_batched_kernel<true, true, 3> : eval_batched_kernel<false, true, 3>;
+  if (minb == 5) return ext ? eval_batched_kernel<true, true, 5> : eval_batched_kernel<false, true, 5>;
+  return ext ? eval_batched_kernel<true, true, 4> : eval_batched_kernel<false, true, 4>;
+}
+sr_status launch_batch_pass(sr_ctx *ctx, bool ext, bool wide, int minb, int smem, const BatchParams &b) {
+  const BatchKernel k = batch_kernel_for(ext, wide, minb);
+  int grid = 0;
+  sr_status st = persistent_grid(ctx, reinterpret_cast<const void *>(k), smem, &grid);
   if (st != SR_OK) return st;
-  int nb = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, eval_batched_kernel<EXT, MINB>, WARPS * 32, smem);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-  if (nb < 1) return fail(ctx, SR_EINVAL, "Lmax too large for shared memory");
-  *grid = nb * ctx->num_sms;
+  k<<<grid, WARPS * 32, smem, ctx->stream>>>(b);
+  ctx->launches += 1;
   return SR_OK;
-}
-
-template <bool EXT>
-sr_status batched_grid(sr_ctx *ctx, int minb, int smem, int *grid) {
-  return minb == 3 ? batched_grid_m<EXT, 3>(ctx, smem, grid)
-                   : (minb == 5 ? batched_grid_m<EXT, 5>(ctx, smem, grid) : batched_grid_m<EXT, 4>(ctx, smem, grid));
-}
-
-template <bool EXT>
-void launch_batched_kernel(int minb, int grid, int smem, cudaStream_t s, const BatchParams &b) {
-  if (minb == 3) eval_batched_kernel<EXT, 3><<<grid, WARPS * 32, smem, s>>>(b);
-  else if (minb == 5) eval_batched_kernel<EXT, 5><<<grid, WARPS * 32, smem, s>>>(b);
-  else eval_batched_kernel<EXT, 4><<<grid, WARPS * 32, smem, s>>>(b);
 }
 
 sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
@@ -1384,16 +1291,13 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
   const int bslots = shallow_slots(maxL, bminb);
   const int smem = WARPS * warp_smem_bytes(bslots, maxL);
   const int smem_deep = slots_for(maxL) > bslots ? WARPS * warp_smem_bytes(slots_for(maxL), maxL) : 0;
-  int grid = 0, grid_ext = 0, grid_deep = 0;
-  sr_status st = batched_grid<false>(ctx, bminb, smem, &grid);
-  if (st != SR_OK) return st;
-  st = batched_grid<true>(ctx, bminb, smem, &grid_ext);
-  if (st != SR_OK) return st;
-  if (smem_deep) {
-    st = batched_grid<true>(ctx, 4, smem_deep, &grid_deep);
-    if (st != SR_OK) return st;
-  }
-  const long long warps = (long long)grid * WARPS;
+  // the cases per item by chunk_ctas' rule, whatever the kernels take
+  const int code = ((maxL * 8 + 15) / 16) * 16;
+  const int cminb = ctx->batched_ctas == 5 && WARPS * (fit_slots(maxL, 5, code) * SLOT_BYTES + code) > smem_target(5)
+                        ? 4
+                        : (ctx->batched_ctas ? ctx->batched_ctas : 4);
+  const long long warps = (long long)chunk_ctas(maxL, cminb) * ctx->num_sms * WARPS;
+  Layout lay = LAY_TABLE;
   const double want = (double)warps * TARGET_ITEMS_PER_WARP;
 
   // chunking per problem: items in proportion to its share of the work
@@ -1434,7 +1338,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
     long long depth2 = 0;  // bytes of the group's tables with compositions
     const size_t off_q = cv.take(256);
     long long items = 0;
-    int corr_chunks = 0, ncorr = 0, progs = 0;
+    int corr_chunks = 0, ncorr = 0, progs = 0, stages = 0;
     for (size_t g = g0; g < g1; ++g) {
       const int i = order[g];
       const sr_problem &q = pr[i];
@@ -1452,7 +1356,9 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
         off_st = cv.take((size_t)nch[i] * 16);
       }
       int ldxt = 0;
-      int xf = use_xform(ctx, q.P, q.nvars, q.N, &ldxt);
+      int xf = lay == LAY_TABLE ? use_xform(ctx, q.P, q.nvars, q.N, &ldxt) : 0;
+      ldxt = (q.N + CPL - 1) / CPL * CPL;
+      const bool stage = !xf && lay != LAY_PLAIN && !rows_are_wide(q.X, q.ldx);
       if (xf == 2) {
         const long long b2 = (long long)xform_rows(q.nvars, 2) * ldxt * 4;
         if (depth2 + b2 > XFORM2_BATCH_BYTES) xf = 1;
@@ -1462,6 +1368,8 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
         const size_t rows = (size_t)xform_rows(q.nvars, xf);
         off_xt = cv.take(rows * ldxt * 4);
         off_xn = cv.take(rows - q.nvars);
+      } else if (stage) {
+        off_xt = cv.take((size_t)q.nvars * ldxt * 4);
       }
       if (bpar) {
         BatchProblem &b = bpar->prob[g - g0];
@@ -1493,7 +1401,10 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
         b.corr_chunk_begin = corr ? corr_chunks : -1;
         b.xform = xf;
         b.xneed = xf ? reinterpret_cast<uint8_t *>(ws + off_xn) : nullptr;
-        if (xf) {
+        b.Xsrc = stage ? q.X : nullptr;
+        b.ldsrc = q.ldx;
+        b.stage_begin = stages;
+        if (xf || stage) {
           b.X = reinterpret_cast<const float *>(ws + off_xt);
           b.ldx = ldxt;
         }
@@ -1501,6 +1412,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       }
       items += (long long)q.P * nch[i];
       progs += q.P;
+      if (stage) stages += stage_blocks(q.nvars, q.N);
       if (corr) {
         corr_chunks += nch[i];
         ++ncorr;
@@ -1515,36 +1427,28 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       bpar->slots = bslots;
       bpar->maxL = maxL;
       bpar->warp_bytes = warp_smem_bytes(bpar->slots, maxL);
-      bpar->deep = 0;
+      bpar->pass = PASS_BASE;
+      bpar->decode_blocks = (progs + DECODE_WARPS - 1) / DECODE_WARPS;
+      bpar->stage_blocks = stages;
       bpar->abort = ctx->abort_flag;
       bpar->err = ctx->dev_words;
     }
     return cv.off;
   };
-  size_t need = 0;
-  for (size_t g0 = 0; g0 < order.size(); g0 += MAX_BATCH) {
-    const size_t g1 = std::min(order.size(), g0 + MAX_BATCH);
-    need = std::max(need, group_bytes(g0, g1, nullptr));
-  }
   if (order.empty()) return SR_OK;
-  st = ensure_workspace(ctx, need);
-  // no room for the variable tables: evaluate without them (the context's
-  // setting comes back when the call returns)
-  struct Restore {
-    sr_ctx *c;
-    int mode;
-    ~Restore() { c->xform = mode; }
-  } restore{ctx, ctx->xform};
-  if (st == SR_ENOMEM && ctx->xform != 0) {
-    ctx->xform = 0;
-    need = 0;
-    for (size_t g0 = 0; g0 < order.size(); g0 += MAX_BATCH) {
-      const size_t g1 = std::min(order.size(), g0 + MAX_BATCH);
-      need = std::max(need, group_bytes(g0, g1, nullptr));
-    }
+  // with less room: without the variable tables, then without copies of X
+  sr_status st = SR_ENOMEM;
+  for (Layout l : {LAY_TABLE, LAY_COPY, LAY_PLAIN}) {
+    lay = l;
+    size_t need = 0;
+    for (size_t g0 = 0; g0 < order.size(); g0 += MAX_BATCH)
+      need = std::max(need, group_bytes(g0, std::min(order.size(), g0 + MAX_BATCH), nullptr));
     st = ensure_workspace(ctx, need);
+    if (st != SR_ENOMEM) break;
   }
   if (st != SR_OK) return st;
+  bool wide = true;
+  for (int i : order) wide = wide && (lay != LAY_PLAIN || rows_are_wide(pr[i].X, pr[i].ldx));
 
   cudaStream_t s = ctx->stream;
   for (size_t g0 = 0; g0 < order.size(); g0 += MAX_BATCH) {
@@ -1558,7 +1462,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       if (b.prob[r].xform)
         SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.prob[r].xneed, 0,
                                            (size_t)(xform_rows(b.prob[r].nvars, b.prob[r].xform) - b.prob[r].nvars), s));
-    decode_batched_kernel<<<(b.total_progs + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
+    decode_batched_kernel<<<b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
                             DECODE_WARPS * decode_warp_bytes(maxL), s>>>(b);
     ctx->launches += 1;
     for (size_t g = g0; g < g1; ++g) {  // the variable tables, from the problems' own X
@@ -1575,17 +1479,22 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       ycenter_batched_kernel<<<corr_blocks, PREP_THREADS, 0, s>>>(b);
       ctx->launches += 2;
     }
-    launch_batched_kernel<false>(bminb, grid, smem, s, b);
-    launch_batched_kernel<true>(bminb, grid_ext, smem, s, b);
-    ctx->launches += 2;
-    if (smem_deep) {
+    if (wide) {
+      st = launch_batch_pass(ctx, false, true, bminb, smem, b);
+      b.pass = PASS_EXT;
+      if (st == SR_OK) st = launch_batch_pass(ctx, true, true, bminb, smem, b);
+    } else {
+      b.pass = PASS_SHALLOW;
+      st = launch_batch_pass(ctx, true, false, 4, smem, b);
+    }
+    if (st == SR_OK && smem_deep) {
       BatchParams bd = b;
-      bd.deep = 1;
+      bd.pass = PASS_DEEP;
       bd.slots = slots_for(maxL);
       bd.warp_bytes = warp_smem_bytes(bd.slots, maxL);
-      launch_batched_kernel<true>(4, grid_deep, smem_deep, s, bd);
-      ctx->launches += 1;
+      st = launch_batch_pass(ctx, true, wide, 4, smem_deep, bd);
     }
+    if (st != SR_OK) return st;
     int maxP = 1;
     for (int r = 0; r < b.nprob; ++r) maxP = b.prob[r].P > maxP ? b.prob[r].P : maxP;
     const int yblocks = std::min((maxP + FINAL_WARPS - 1) / FINAL_WARPS, 65535);
@@ -1684,13 +1593,10 @@ sr_status sr_reserve(sr_ctx *ctx, int P, int Lmax, int N) {
   if (!ctx || P < 0 || Lmax < 1 || Lmax > SR_MAX_LMAX || N < 1) return SR_EINVAL;
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
   size_t need = 0;
-  for (int mode = 0; mode < 4; ++mode) {
+  for (int nv = 1; nv <= SR_MAX_VARS; ++nv) {  // the table's size depends on the variable count
     Plan pl;
-    for (int nv = 1; nv <= SR_MAX_VARS; ++nv) {  // the table's size depends on the variable count
-      sr_status st = make_plan(ctx, mode, P, Lmax, N, &pl, nv);
-      if (st != SR_OK) return st;
-      need = pl.bytes > need ? pl.bytes : need;
-    }
+    make_plan(ctx, P, Lmax, N, &pl, nv, false, LAY_TABLE);
+    need = pl.bytes > need ? pl.bytes : need;
   }
   return ensure_workspace(ctx, need);
 }
@@ -1764,8 +1670,7 @@ extern "C" sr_status sr_eval_noalloc(void *cuda_stream, const uint8_t *programs,
   // fewer work items and partial records
   Plan pl;
   for (;;) {
-    st = make_plan(&local, mode, P, Lmax, N, &pl);
-    if (st != SR_OK) return st;
+    make_plan(&local, P, Lmax, N, &pl, nvars, false, LAY_PLAIN);  // (a copy of X only where it fits as well)
     if (pl.bytes <= NOALLOC_SCRATCH_BYTES) break;
     if (local.num_sms == 1) return SR_ENOMEM;  // does not fit even on one SM
     local.num_sms = local.num_sms / 2 > 0 ? local.num_sms / 2 : 1;
@@ -1775,6 +1680,7 @@ extern "C" sr_status sr_eval_noalloc(void *cuda_stream, const uint8_t *programs,
   if (st != SR_OK) return st;
   local.ws = static_cast<char *>(scratch);
   local.ws_bytes = NOALLOC_SCRATCH_BYTES;
+  local.ws_fixed = true;
   return launch_eval(&local, mode, programs, lengths, consts, P, Lmax, K, X, y, nvars, N, ldx,
                      fitness, prog_flags, nullptr, 0);
 }

@@ -125,6 +125,7 @@ enum Op : uint32_t {
   OP_CDIV,
   OP_CRSUB,     // top = c_k - top
   OP_CRDIV,     // top = c_k / top
+  OP_END,       // the program is done (appended by the evaluation kernels)
 };
 
 __device__ __forceinline__ uint32_t ins_op(uint2 w) { return w.x & 0xffu; }
