@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "sr_common.cuh"
+#include "sr_decode.cuh"
 #include "sr_interp.cuh"
 #include "sr_vm.cuh"
 
@@ -210,8 +211,13 @@ __device__ void stage_rows(const EvalParams &p, int block) {
 __global__ void decode_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
   const int dblocks = (p.P + DECODE_WARPS - 1) / DECODE_WARPS;
-  if ((int)blockIdx.x >= dblocks) stage_rows(p, blockIdx.x - dblocks);
-  else decode_warp(decode_args(p, p.slots, p.queue + 4), p.P, dsm);
+  if ((int)blockIdx.x >= dblocks) {
+    stage_rows(p, blockIdx.x - dblocks);
+    return;
+  }
+  const int warp = threadIdx.x >> 5, prog = blockIdx.x * DECODE_WARPS + warp;
+  if (prog < p.P)
+    decode_eval_warp(decode_args(p, p.slots, p.queue + 4), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
 }
 
 // The variable table of an evaluation with transforms (DecodeArgs::xform):
@@ -660,8 +666,8 @@ __global__ void decode_batched_kernel(const __grid_constant__ BatchParams b) {
   }
   EvalParams p = view(b.prob[lo]);
   p.queue = b.queue;
-  decode_warp_one(decode_args(p, b.slots, b.queue + 4), g - b.prob[lo].prog_begin,
-                  dsm + (size_t)warp * decode_warp_bytes(b.maxL));
+  decode_eval_warp(decode_args(p, b.slots, b.queue + 4), g - b.prob[lo].prog_begin,
+                   dsm + (size_t)warp * decode_scratch_bytes(b.maxL));
 }
 
 // Work items of every problem come from one atomic counter: problem q owns
@@ -1206,7 +1212,7 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   if (st != SR_OK) return st;
   const int stage = pl.stage ? stage_blocks(nvars, N) : 0;
   decode_kernel<<<(P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
-                  DECODE_WARPS * decode_warp_bytes(Lmax), s>>>(ep);
+                  DECODE_WARPS * decode_scratch_bytes(Lmax), s>>>(ep);
   ctx->launches += 1;
   if (pl.xform) {
     const dim3 g((unsigned)((N + XF_THREADS * 4 - 1) / (XF_THREADS * 4)), (unsigned)xform_rows(nvars, pl.xform));
@@ -1463,7 +1469,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
         SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.prob[r].xneed, 0,
                                            (size_t)(xform_rows(b.prob[r].nvars, b.prob[r].xform) - b.prob[r].nvars), s));
     decode_batched_kernel<<<b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
-                            DECODE_WARPS * decode_warp_bytes(maxL), s>>>(b);
+                            DECODE_WARPS * decode_scratch_bytes(maxL), s>>>(b);
     ctx->launches += 1;
     for (size_t g = g0; g < g1; ++g) {  // the variable tables, from the problems' own X
       const BatchProblem &q = b.prob[g - g0];
