@@ -185,8 +185,6 @@ __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_s
   a.max_slots = slots_for(p.Lmax);
   a.cap_slots = cap_slots;
   a.deep_count = deep_count;
-  a.fold = 1;  // constant-only subtrees are evaluated once, in the decoder
-  a.adj_info = 0;
   a.xform = p.xform;
   a.xneed = p.xneed;
   return a;
