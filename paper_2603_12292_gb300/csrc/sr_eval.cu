@@ -107,6 +107,8 @@ struct EvalParams {
   int xform = 0;           // >= 1: X is the variable table of this depth (DecodeArgs::xform)
   const float *Xsrc = nullptr;  // rows to copy into X (the caller's X, not laid out for 256-bit loads), or NULL
   long long ldsrc = 0;
+  double *ysum = nullptr;    // [nchunks][2] chunk sums and counts of y, where the target is centred, or NULL
+  int finite_only = 0;       // 1: over the finite targets (Eq. 2)
   uint8_t *xneed = nullptr;  // the transforms some program reads
 };
 
@@ -165,6 +167,95 @@ __device__ __forceinline__ float4 ldx4(const float *p) {
   return __ldg(reinterpret_cast<const float4 *>(p));
 }
 
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+  return v;
+}
+
+// ---------------------------------------------------------------- target prep (1 - r^2)
+// Two passes over y: the sum of every chunk, then the centred target with its
+// sums.  They run as blocks of the decode launch and of the table's launch: a
+// block per chunk leaves most of the GPU idle (11 + 18 us for 23 chunks of 4,352
+// cases, 22 + 32 for 10 of 13,312), and both are done before those launches are.
+constexpr int PREP_THREADS = 512;
+
+__device__ double block_sum(double v, double *red) {
+  v = warp_sum(v);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
+  __syncthreads();
+  return s;  // valid in thread 0
+}
+
+// FP64 sum and count of one chunk of y: every value, or (finite_only) the
+// finite ones.  ysum [nchunks][2].
+__device__ void ysum_chunk(const float *__restrict__ y, int N, int chunk, int c, bool finite_only,
+                           double *ysum, double *red) {
+  const int beg = c * chunk, end = min(N, beg + chunk);
+  double a = 0.0, n = 0.0;
+  for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
+    const float v = __ldg(y + i);
+    if (!finite_only || isfinite(v)) {
+      a += (double)v;
+      n += 1.0;
+    }
+  }
+  a = block_sum(a, red);
+  n = block_sum(n, red);
+  if (threadIdx.x == 0) {
+    ysum[2 * c] = a;
+    ysum[2 * c + 1] = n;
+  }
+}
+
+// ybar = (sum of the chunk sums) / (their count), chunks in order; then
+// yc = fl32(y - ybar) on one chunk (NaN at invalid targets when
+// nan_invalid) with the chunk's FP64 sum and sum of squares of yc
+__device__ void ycenter_chunk(const float *__restrict__ y, int N, int chunk, int nchunks, int c,
+                              const double *ysum, bool nan_invalid, float *yc, double *ychunk,
+                              double *red) {
+  __shared__ double ybar_s;
+  if (threadIdx.x == 0) {
+    double t = 0.0, n = 0.0;
+    for (int k = 0; k < nchunks; ++k) {
+      t += ysum[2 * k];
+      n += ysum[2 * k + 1];
+    }
+    ybar_s = n > 0.0 ? t / n : 0.0;
+  }
+  __syncthreads();
+  const double ybar = ybar_s;
+  const int beg = c * chunk, end = min(N, beg + chunk);
+  double a = 0.0, b = 0.0;
+  for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
+    const float yi = y[i];
+    if (nan_invalid && !isfinite(yi)) {
+      yc[i] = __int_as_float(0x7fc00000);
+      continue;
+    }
+    const float v = (float)((double)yi - ybar);
+    yc[i] = v;
+    a += (double)v;
+    b += (double)v * (double)v;
+  }
+  if (c == nchunks - 1) {
+    const int padded = (N + STEP - 1) / STEP * STEP;
+    for (int i = N + threadIdx.x; i < padded; i += blockDim.x) yc[i] = 0.0f;
+  }
+  a = block_sum(a, red);
+  b = block_sum(b, red);
+  if (threadIdx.x == 0) {
+    ychunk[2 * c] = a;
+    ychunk[2 * c + 1] = b;
+  }
+}
+
+
 // ---------------------------------------------------------------- decode pre-pass
 // cap_slots: programs that need more get NCODE_DEEP, counted in deep_count
 __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_slots,
@@ -204,16 +295,23 @@ __device__ void stage_rows(const EvalParams &p, int block) {
     *reinterpret_cast<float4 *>(dst + i) = ldx4(src + i);  // i + 3 < both strides: multiples of 4, >= N
 }
 
-// one warp per program, scratch in shared memory (decode_warp); the blocks
-// after those copy X where it is not laid out for 256-bit loads
-__global__ void decode_kernel(EvalParams p) {
+// The first blocks sum the chunks of y where the target is centred, the next
+// decode (one warp per program, scratch in shared memory), the last copy X where
+// it is not laid out for 256-bit loads.
+__global__ void __launch_bounds__(DECODE_WARPS * 32) decode_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  const int dblocks = (p.P + DECODE_WARPS - 1) / DECODE_WARPS;
-  if ((int)blockIdx.x >= dblocks) {
-    stage_rows(p, blockIdx.x - dblocks);
+  __shared__ double red[DECODE_WARPS];
+  const int yblocks = p.ysum ? p.nchunks : 0, dblocks = (p.P + DECODE_WARPS - 1) / DECODE_WARPS;
+  const int block = (int)blockIdx.x - yblocks;
+  if (block < 0) {
+    ysum_chunk(p.y, p.N, p.chunk, blockIdx.x, p.finite_only != 0, p.ysum, red);
     return;
   }
-  const int warp = threadIdx.x >> 5, prog = blockIdx.x * DECODE_WARPS + warp;
+  if (block >= dblocks) {
+    stage_rows(p, block - dblocks);
+    return;
+  }
+  const int warp = threadIdx.x >> 5, prog = block * DECODE_WARPS + warp;
   if (prog < p.P)
     decode_eval_warp(decode_args(p, p.slots, p.queue + 4), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
 }
@@ -222,34 +320,77 @@ __global__ void decode_kernel(EvalParams p) {
 // row j < nvars is x_j, row xform_row(nvars, u, j) is u(x_j) and row
 // xform_row2(nvars, u, v, j) is u(v(x_j)), for the rows some program reads
 // (xneed, marked by the decoder), by the interpreter's own FP32 functions
-// (fold_op), so a program reads the bits its own per-case evaluation would
-// give.  Blocks: (case group of XF_THREADS * 4 cases, row).
-constexpr int XF_THREADS = 256;
-__global__ void __launch_bounds__(XF_THREADS)
-    xform_kernel(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt,
-                 const uint8_t *__restrict__ xneed, float *__restrict__ xt) {
-  const int r = blockIdx.y;
-  if (r >= nvars && !xneed[r - nvars]) return;
-  const int c = (blockIdx.x * XF_THREADS + threadIdx.x) * 4;
-  if (c >= N) return;  // c + 3 < ldx and < ldxt: both are multiples of 4 and >= N
-  const int r2 = nvars * (1 + UNARY_ALL);  // first composition row
-  int u = -1, v = -1, j = r;
-  if (r >= r2) {
-    const int k = (r - r2) / nvars;
-    j = (r - r2) % nvars;
-    u = TOK_SIN + k / XFORM_BASE;
-    v = TOK_SIN + k % XFORM_BASE;
-  } else if (r >= nvars) {
-    u = TOK_SIN + (r - nvars) / nvars;
-    j = (r - nvars) % nvars;
+// (fold_op's), so a program reads the bits its own per-case evaluation would
+// give.  Blocks: (XF_THREADS * 4 cases, variable and part): part 0 the variable
+// and the operators beyond the base ones, part 1 + v the base operator v and its
+// compositions, which read v(x_j) from registers.  What bounds it: issue slots.
+// A block per row, each value through a call of fold_op, computed v(x_j) seven
+// times: 118 us for 490 rows of 100,003 cases, now 40.
+constexpr int XF_THREADS = 256, XF_PARTS = 1 + XFORM_BASE;
+static __device__ __noinline__ float4 unary4(int tok, float4 x) {
+#define SR_EACH(f) make_float4(f(x.x), f(x.y), f(x.z), f(x.w))
+  switch (tok) {
+    case TOK_SIN: return SR_EACH(f_sin);
+    case TOK_COS: return SR_EACH(f_cos);
+    case TOK_EXP: return SR_EACH(op_exp);
+    case TOK_LOG: return SR_EACH(op_log);
+    case TOK_SQRT: return SR_EACH(f_sqrt);
+    case TOK_SQ: return make_float4(__fmul_rn(x.x, x.x), __fmul_rn(x.y, x.y), __fmul_rn(x.z, x.z), __fmul_rn(x.w, x.w));
+    default:
+      return make_float4(fold_op(tok, x.x, 0.f), fold_op(tok, x.y, 0.f), fold_op(tok, x.z, 0.f), fold_op(tok, x.w, 0.f));
   }
-  float4 x = ldx4(X + (size_t)j * ldx + c);
-  if (v >= 0)
-    x = make_float4(fold_op(v, x.x, 0.f), fold_op(v, x.y, 0.f), fold_op(v, x.z, 0.f), fold_op(v, x.w, 0.f));
-  if (u >= 0)
-    x = make_float4(fold_op(u, x.x, 0.f), fold_op(u, x.y, 0.f), fold_op(u, x.z, 0.f), fold_op(u, x.w, 0.f));
-  *reinterpret_cast<float4 *>(xt + (size_t)r * ldxt + c) = x;
+#undef SR_EACH
 }
+__device__ void xform_block(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt, int depth,
+                            const uint8_t *__restrict__ xneed, float *__restrict__ xt, int block, int j, int part) {
+  const int c = (block * XF_THREADS + threadIdx.x) * 4;
+  if (c >= N) return;  // c + 3 < ldx and < ldxt: both are multiples of 4 and >= N
+  const float4 x = ldx4(X + (size_t)j * ldx + c);
+  auto put = [&](int row, float4 v) { *reinterpret_cast<float4 *>(xt + (size_t)row * ldxt + c) = v; };
+  auto needed = [&](int row) { return xneed[row - nvars] != 0; };
+  if (part == 0) {
+    put(j, x);
+    for (int u = TOK_SQ + 1; u <= TOK_TANH; ++u)
+      if (needed(xform_row(nvars, u, j))) put(xform_row(nvars, u, j), unary4(u, x));
+    return;
+  }
+  const int v = TOK_SIN + part - 1;
+  bool any = needed(xform_row(nvars, v, j));
+  if (depth > 1)
+    for (int u = TOK_SIN; u <= TOK_SQ; ++u) any = any || needed(xform_row2(nvars, u, v, j));
+  if (!any) return;
+  const float4 y = unary4(v, x);
+  if (needed(xform_row(nvars, v, j))) put(xform_row(nvars, v, j), y);
+  if (depth > 1)
+    for (int u = TOK_SIN; u <= TOK_SQ; ++u)
+      if (needed(xform_row2(nvars, u, v, j))) put(xform_row2(nvars, u, v, j), unary4(u, y));
+}
+struct CenterParams {
+  const float *y;
+  int N, chunk, nchunks, nan_invalid;
+  const double *ysum;
+  float *yc;
+  double *ychunk;
+};
+__global__ void __launch_bounds__(PREP_THREADS) ycenter_kernel(CenterParams y) {
+  __shared__ double red[PREP_THREADS / 32];
+  ycenter_chunk(y.y, y.N, y.chunk, y.nchunks, blockIdx.x, y.ysum, y.nan_invalid != 0, y.yc, y.ychunk, red);
+}
+// The first yblocks blocks centre the target, one chunk each.
+__global__ void __launch_bounds__(XF_THREADS)
+    xform_kernel(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt, int depth,
+                 const uint8_t *__restrict__ xneed, float *__restrict__ xt, int yblocks, CenterParams y) {
+  __shared__ double red[XF_THREADS / 32];
+  const int block = (int)blockIdx.x - yblocks, per_part = (N + XF_THREADS * 4 - 1) / (XF_THREADS * 4);
+  if (block < 0) {
+    ycenter_chunk(y.y, y.N, y.chunk, y.nchunks, blockIdx.x, y.ysum, y.nan_invalid != 0, y.yc, y.ychunk, red);
+    return;
+  }
+  const int part = block / per_part;
+  xform_block(X, ldx, nvars, N, ldxt, depth, xneed, xt, block % per_part, part / XF_PARTS, part % XF_PARTS);
+}
+static_assert(DECODE_WARPS * 8192 <= 48 * 1024, "the decode launch needs no shared memory opt-in");
+inline int xform_blocks(int nvars, int N) { return nvars * XF_PARTS * ((N + XF_THREADS * 4 - 1) / (XF_THREADS * 4)); }
 
 // ---------------------------------------------------------------- reductions
 struct Kahan {
@@ -262,12 +403,6 @@ struct Kahan {
   }
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  return v;
-}
 
 __device__ __forceinline__ float sel(bool ok, float v) { return ok ? v : 0.0f; }
 
@@ -607,7 +742,8 @@ struct BatchParams {
   int slots;
   int maxL;                   // the largest Lmax of the batch
   int pass;                   // as EvalParams::pass
-  int decode_blocks, stage_blocks;  // blocks of the decode launch that decode, then those that copy X
+  // blocks of the decode launch: those that sum chunks of y, that decode, that copy X
+  int ysum_blocks, decode_blocks, stage_blocks;
   const int32_t *abort;       // as EvalParams::abort
   unsigned *err;
 };
@@ -641,12 +777,26 @@ __device__ __forceinline__ EvalParams view(const BatchProblem &q) {
   return p;
 }
 
+// the problem whose target chunk a block of the target's launches takes
+__device__ __forceinline__ int corr_problem_of_block(const BatchParams &b) {
+  int r = 0;
+  while (r + 1 < b.ncorr && b.prob[b.corr_list[r + 1]].corr_chunk_begin <= (int)blockIdx.x) ++r;
+  return b.corr_list[r];
+}
+
 // a warp per program of every problem in the batch (shared regions sized
 // for the batch's largest Lmax, b.maxL)
-__global__ void decode_batched_kernel(const __grid_constant__ BatchParams b) {
+__global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char dsm[];
-  if ((int)blockIdx.x >= b.decode_blocks) {
-    const int r = (int)blockIdx.x - b.decode_blocks;
+  __shared__ double red[DECODE_WARPS];
+  const int block = (int)blockIdx.x - b.ysum_blocks;
+  if (block < 0) {
+    const BatchProblem &q = b.prob[corr_problem_of_block(b)];
+    ysum_chunk(q.y, q.N, q.chunk, (int)blockIdx.x - q.corr_chunk_begin, false, q.ysum, red);
+    return;
+  }
+  if (block >= b.decode_blocks) {
+    const int r = block - b.decode_blocks;
     int i = 0;
     while (i + 1 < b.nprob && b.prob[i + 1].stage_begin <= r) ++i;
     const EvalParams p = view(b.prob[i]);
@@ -654,7 +804,7 @@ __global__ void decode_batched_kernel(const __grid_constant__ BatchParams b) {
     return;
   }
   const int warp = threadIdx.x >> 5;
-  const int g = blockIdx.x * (blockDim.x >> 5) + warp;
+  const int g = block * DECODE_WARPS + warp;
   if (g >= b.total_progs) return;
   int lo = 0, hi = b.nprob - 1;
   while (lo < hi) {
@@ -701,104 +851,32 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __
   }
 }
 
-// ---------------------------------------------------------------- target prep (1 - r^2)
-constexpr int PREP_THREADS = 512;
-
-__device__ double block_sum(double v, double *red) {
-  v = warp_sum(v);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-  __syncthreads();
-  return s;  // valid in thread 0
-}
-
-// FP64 sum and count of one chunk of y: every value, or (finite_only) the
-// finite ones.  ysum [nchunks][2].
-__device__ void ysum_chunk(const float *__restrict__ y, int N, int chunk, int c, bool finite_only,
-                           double *ysum, double *red) {
-  const int beg = c * chunk, end = min(N, beg + chunk);
-  double a = 0.0, n = 0.0;
-  for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    const float v = y[i];
-    if (!finite_only || isfinite(v)) {
-      a += (double)v;
-      n += 1.0;
-    }
-  }
-  a = block_sum(a, red);
-  n = block_sum(n, red);
-  if (threadIdx.x == 0) {
-    ysum[2 * c] = a;
-    ysum[2 * c + 1] = n;
-  }
-}
-
-__global__ void __launch_bounds__(PREP_THREADS) ysum_kernel(const float *__restrict__ y, int N, int chunk,
-                                                            int finite_only, double *ysum) {
-  __shared__ double red[PREP_THREADS / 32];
-  ysum_chunk(y, N, chunk, blockIdx.x, finite_only != 0, ysum, red);
-}
-
-// ybar = (sum of the chunk sums) / (their count), chunks in order; then
-// yc = fl32(y - ybar) on one chunk (NaN at invalid targets when
-// nan_invalid) with the chunk's FP64 sum and sum of squares of yc
-__device__ void ycenter_chunk(const float *__restrict__ y, int N, int chunk, int nchunks, int c,
-                              const double *ysum, bool nan_invalid, float *yc, double *ychunk,
-                              double *red) {
-  __shared__ double ybar_s;
-  if (threadIdx.x == 0) {
-    double t = 0.0, n = 0.0;
-    for (int k = 0; k < nchunks; ++k) {
-      t += ysum[2 * k];
-      n += ysum[2 * k + 1];
-    }
-    ybar_s = n > 0.0 ? t / n : 0.0;
-  }
-  __syncthreads();
-  const double ybar = ybar_s;
-  const int beg = c * chunk, end = min(N, beg + chunk);
-  double a = 0.0, b = 0.0;
-  for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    const float yi = y[i];
-    if (nan_invalid && !isfinite(yi)) {
-      yc[i] = __int_as_float(0x7fc00000);
-      continue;
-    }
-    const float v = (float)((double)yi - ybar);
-    yc[i] = v;
-    a += (double)v;
-    b += (double)v * (double)v;
-  }
-  if (c == nchunks - 1) {
-    const int padded = (N + STEP - 1) / STEP * STEP;
-    for (int i = N + threadIdx.x; i < padded; i += blockDim.x) yc[i] = 0.0f;
-  }
-  a = block_sum(a, red);
-  b = block_sum(b, red);
-  if (threadIdx.x == 0) {
-    ychunk[2 * c] = a;
-    ychunk[2 * c + 1] = b;
-  }
-}
-
-__global__ void __launch_bounds__(PREP_THREADS) ycenter_kernel(const float *__restrict__ y, int N,
-                                                               int chunk, int nchunks,
-                                                               const double *ysum, int nan_invalid,
-                                                               float *yc, double *ychunk) {
-  __shared__ double red[PREP_THREADS / 32];
-  ycenter_chunk(y, N, chunk, nchunks, blockIdx.x, ysum, nan_invalid != 0, yc, ychunk, red);
-}
-
 // ---------------------------------------------------------------- finalize
-// The merges below run with a warp per program: lane l takes chunks l,
-// l + 32, ...; every sum over chunks is a per-lane sum followed by a fixed
-// xor-butterfly reduction (warp_sum), so the result is deterministic and
-// the same on every lane.  (A thread per program ran the FP64 chain of all
-// chunks serially: 0.7 % of a 4,096 x 100,000 generation.)
+// The merges below run with a group of lanes per program, a power of two by the
+// number of chunks (about four chunks a lane): lane l of the group takes chunks
+// l, l + lanes, ...; every sum over chunks is a per-lane sum followed by a fixed
+// xor-butterfly over the group, so the result is deterministic and the same on
+// every lane.  What bounds it: the FP64 pipe (two lanes an SM), which a warp per
+// program kept busy with idle lanes.  Before -> now (us): 64 small problems,
+// 22,000 programs of 1 to 40 chunks, 106 -> 21; 8,192 programs of 10 chunks 54 -> 14;
+// 4,096 of 23 33 -> 16; 1,500 of 56 27 -> 23.
+__host__ __device__ inline int merge_lanes(int nchunks) {
+  int g = 1;
+  while (g < 32 && g * 4 < nchunks) g *= 2;
+  return g;
+}
+struct Group {
+  int lane, lanes;
+  unsigned mask;
+  __device__ __forceinline__ double sum(double v) const {
+    for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+  }
+};
+__device__ __forceinline__ Group group_of(int lanes) {
+  const int l = threadIdx.x & 31;
+  return Group{l & (lanes - 1), lanes, (lanes == 32 ? FULL : (1u << lanes) - 1u) << (l & ~(lanes - 1))};
+}
 
 // 1 - r^2 of one program from its chunk records.
 // chunk c: n_c cases, shift s_c, S1 = sum d, S2 = sum d^2, S3 = sum d yc with
@@ -806,29 +884,31 @@ __global__ void __launch_bounds__(PREP_THREADS) ycenter_kernel(const float *__re
 // merged (Chan et al.): Shh = sum M2_c + n_c (m_c - m)^2.
 // sum yhat*yc = sum (S3_c + s_c Yc_c); Shy = that - m * Y1; Syy = Y2 - Y1^2/N.
 __device__ double corr_fitness(const double *rec, const double *ychunk, int Nc, int chunk,
-                               int nchunks, int lane) {
+                               int nchunks, const Group &g) {
   const double N = (double)Nc;
   double y1 = 0.0, y2 = 0.0, tot = 0.0;
-  for (int c = lane; c < nchunks; c += 32) {
+  for (int c = g.lane; c < nchunks; c += g.lanes) {
     y1 += ychunk[2 * c];
     y2 += ychunk[2 * c + 1];
     const double nc = (double)min(chunk, Nc - c * chunk);
     tot += nc * rec[c * PSTRIDE + 1] + rec[c * PSTRIDE + 2];
   }
-  y1 = warp_sum(y1);
-  y2 = warp_sum(y2);
-  const double m = warp_sum(tot) / N;
-  double shh = 0.0, g = 0.0;
-  for (int c = lane; c < nchunks; c += 32) {
-    const double nc = (double)min(chunk, Nc - c * chunk);
+  y1 = g.sum(y1);
+  y2 = g.sum(y2);
+  const double m = g.sum(tot) / N;
+  // every chunk but the last has `chunk` cases: one reciprocal instead of two divisions a chunk
+  const double inv_full = 1.0 / (double)chunk, inv_last = 1.0 / (double)(Nc - (nchunks - 1) * chunk);
+  double shh = 0.0, cross = 0.0;
+  for (int c = g.lane; c < nchunks; c += g.lanes) {
+    const double nc = (double)min(chunk, Nc - c * chunk), inv = c == nchunks - 1 ? inv_last : inv_full;
     const double s = rec[c * PSTRIDE + 1], a = rec[c * PSTRIDE + 2];
     const double b = rec[c * PSTRIDE + 3], d = rec[c * PSTRIDE + 4];
-    const double mc = s + a / nc;
-    shh += (b - a * a / nc) + nc * (mc - m) * (mc - m);
-    g += d + s * ychunk[2 * c];
+    const double mc = s + a * inv;
+    shh += (b - a * a * inv) + nc * (mc - m) * (mc - m);
+    cross += d + s * ychunk[2 * c];
   }
-  shh = warp_sum(shh);
-  const double shy = warp_sum(g) - m * y1;
+  shh = g.sum(shh);
+  const double shy = g.sum(cross) - m * y1;
   const double syy = y2 - y1 * y1 / N;
   double fit = 1.0;
   if (isfinite(shh) && isfinite(shy) && isfinite(syy) && shh > 0.0 && syy > 0.0 && Nc >= 2) {
@@ -845,9 +925,9 @@ __device__ double corr_fitness(const double *rec, const double *ychunk, int Nc, 
 // n_c = cases - c1 - c2.  Shh merges the chunks by Chan et al.; e shares one
 // centre, so See = E2 - E1^2 / n; Seh = sum (X_c + s_c E1_c) - m E1.
 __device__ double r4_score(const double *rec, int Nc, int chunk, int nchunks, double M, double *c1o,
-                           double *c2o, int lane) {
+                           double *c2o, const Group &g) {
   double c1 = 0.0, c2 = 0.0, n = 0.0, tot = 0.0, e1 = 0.0, e2 = 0.0;
-  for (int c = lane; c < nchunks; c += 32) {
+  for (int c = g.lane; c < nchunks; c += g.lanes) {
     const double *r = rec + c * PSTRIDE;
     const double nv = (double)min(chunk, Nc - c * chunk) - r[6] - r[7];
     c1 += r[6];
@@ -857,17 +937,17 @@ __device__ double r4_score(const double *rec, int Nc, int chunk, int nchunks, do
     e1 += r[4];
     e2 += r[5];
   }
-  c1 = warp_sum(c1);
-  c2 = warp_sum(c2);
-  n = warp_sum(n);
-  tot = warp_sum(tot);
-  e1 = warp_sum(e1);
-  e2 = warp_sum(e2);
+  c1 = g.sum(c1);
+  c2 = g.sum(c2);
+  n = g.sum(n);
+  tot = g.sum(tot);
+  e1 = g.sum(e1);
+  e2 = g.sum(e2);
   double r2 = 0.0;
   if (n >= 2.0) {
     const double m = tot / n;
     double shh = 0.0, seh = 0.0;
-    for (int c = lane; c < nchunks; c += 32) {
+    for (int c = g.lane; c < nchunks; c += g.lanes) {
       const double *r = rec + c * PSTRIDE;
       const double nv = (double)min(chunk, Nc - c * chunk) - r[6] - r[7];
       if (nv <= 0.0) continue;
@@ -875,8 +955,8 @@ __device__ double r4_score(const double *rec, int Nc, int chunk, int nchunks, do
       shh += (r[2] - r[1] * r[1] / nv) + nv * (mc - m) * (mc - m);
       seh += r[3] + r[0] * r[4];
     }
-    shh = warp_sum(shh);
-    seh = warp_sum(seh) - m * e1;
+    shh = g.sum(shh);
+    seh = g.sum(seh) - m * e1;
     const double see = e2 - e1 * e1 / n;
     if (isfinite(shh) && isfinite(seh) && isfinite(see) && shh > 0.0 && see > 0.0) {
       r2 = (seh * seh) / (shh * see);
@@ -889,30 +969,30 @@ __device__ double r4_score(const double *rec, int Nc, int chunk, int nchunks, do
 }
 
 // fitness of program p from its partial records (mode picks the outputs);
-// called by all 32 lanes of a warp, lane 0 writes
+// called by all lanes of a group, lane 0 writes
 __device__ void finalize_one(int mode, const double *partials, const int32_t *flags,
                              const double *ychunk, int P, int N, int chunk, int nchunks,
-                             double *fitness, int p, int lane, int M = 0, int32_t *counts = nullptr) {
+                             double *fitness, int p, const Group &g, int M = 0, int32_t *counts = nullptr) {
   const double INF = __longlong_as_double(0x7ff0000000000000ll);
   if (mode == MODE_R4 || mode == MODE_P2P) {
     double c1 = 0.0, c2 = 0.0, sc = -INF;
     if (!flags[p]) {
       const double *rec = partials + (size_t)p * nchunks * PSTRIDE;
       if (mode == MODE_R4) {
-        sc = r4_score(rec, N, chunk, nchunks, (double)M, &c1, &c2, lane);
+        sc = r4_score(rec, N, chunk, nchunks, (double)M, &c1, &c2, g);
       } else {
         sc = 0.0;
-        for (int c = lane; c < nchunks; c += 32) {
+        for (int c = g.lane; c < nchunks; c += g.lanes) {
           sc += rec[c * PSTRIDE];
           c1 += rec[c * PSTRIDE + 6];
           c2 += rec[c * PSTRIDE + 7];
         }
-        sc = warp_sum(sc);  // integers below 2^53: exact in any order
-        c1 = warp_sum(c1);
-        c2 = warp_sum(c2);
+        sc = g.sum(sc);  // integers below 2^53: exact in any order
+        c1 = g.sum(c1);
+        c2 = g.sum(c2);
       }
     }
-    if (lane == 0) {
+    if (g.lane == 0) {
       fitness[p] = sc;
       if (counts) {
         counts[2 * p] = (int32_t)c1;
@@ -924,20 +1004,20 @@ __device__ void finalize_one(int mode, const double *partials, const int32_t *fl
   double *mse_out = fitness;
   double *corr_out = mode == MODE_BOTH ? fitness + P : fitness;
   if (flags[p]) {
-    if (lane == 0 && mode != MODE_CORR) mse_out[p] = INF;
-    if (lane == 0 && mode != MODE_MSE) corr_out[p] = INF;
+    if (g.lane == 0 && mode != MODE_CORR) mse_out[p] = INF;
+    if (g.lane == 0 && mode != MODE_MSE) corr_out[p] = INF;
     return;
   }
   const double *rec = partials + (size_t)p * nchunks * PSTRIDE;
   if (mode != MODE_CORR) {
     double se = 0.0;
-    for (int c = lane; c < nchunks; c += 32) se += rec[c * PSTRIDE];
-    se = warp_sum(se);
-    if (lane == 0) mse_out[p] = isfinite(se) ? se / (double)N : INF;
+    for (int c = g.lane; c < nchunks; c += g.lanes) se += rec[c * PSTRIDE];
+    se = g.sum(se);
+    if (g.lane == 0) mse_out[p] = isfinite(se) ? se / (double)N : INF;
   }
   if (mode != MODE_MSE) {
-    const double f = corr_fitness(rec, ychunk, N, chunk, nchunks, lane);
-    if (lane == 0) corr_out[p] = f;
+    const double f = corr_fitness(rec, ychunk, N, chunk, nchunks, g);
+    if (g.lane == 0) corr_out[p] = f;
   }
 }
 
@@ -951,30 +1031,18 @@ struct FinalParams {
   int32_t *counts;  // Beagle scores: [P][2] (c1, c2) or NULL
 };
 
-// a warp per program, FINAL_WARPS programs per block
-constexpr int FINAL_WARPS = 4;
+constexpr int FINAL_THREADS = 128;
 
-__global__ void finalize_kernel(FinalParams f) {
-  const int p = blockIdx.x * FINAL_WARPS + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(FINAL_THREADS) finalize_kernel(FinalParams f) {
+  const int lanes = merge_lanes(f.nchunks), p = (blockIdx.x * FINAL_THREADS + threadIdx.x) / lanes;
   if (p >= f.P) return;
-  finalize_one(f.mode, f.partials, f.flags, f.ychunk, f.P, f.N, f.chunk, f.nchunks, f.fitness, p,
-               threadIdx.x & 31, f.M, f.counts);
+  finalize_one(f.mode, f.partials, f.flags, f.ychunk, f.P, f.N, f.chunk, f.nchunks, f.fitness, p, group_of(lanes), f.M,
+               f.counts);
 }
 
 // ---------------------------------------------------------------- batched prep / finalize
 // one block per (problem, chunk) of the problems that need the centred
-// target: the chunk sums of y, then (next launch) the centred target
-__device__ __forceinline__ int corr_problem_of_block(const BatchParams &b) {
-  int r = 0;
-  while (r + 1 < b.ncorr && b.prob[b.corr_list[r + 1]].corr_chunk_begin <= (int)blockIdx.x) ++r;
-  return b.corr_list[r];
-}
-
-__global__ void __launch_bounds__(PREP_THREADS) ysum_batched_kernel(const __grid_constant__ BatchParams b) {
-  __shared__ double red[PREP_THREADS / 32];
-  const BatchProblem &q = b.prob[corr_problem_of_block(b)];
-  ysum_chunk(q.y, q.N, q.chunk, (int)blockIdx.x - q.corr_chunk_begin, false, q.ysum, red);
-}
+// target (its chunk sums come from the decode launch)
 
 __global__ void __launch_bounds__(PREP_THREADS) ycenter_batched_kernel(const __grid_constant__ BatchParams b) {
   __shared__ double red[PREP_THREADS / 32];
@@ -983,12 +1051,13 @@ __global__ void __launch_bounds__(PREP_THREADS) ycenter_batched_kernel(const __g
                 q.ychunk, red);
 }
 
-// blocks (problem, FINAL_WARPS programs of it), a warp per program
-__global__ void finalize_batched_kernel(const __grid_constant__ BatchParams b) {
+// blocks (problem, FINAL_THREADS / merge_lanes programs of it)
+__global__ void __launch_bounds__(FINAL_THREADS) finalize_batched_kernel(const __grid_constant__ BatchParams b) {
   const BatchProblem &q = b.prob[blockIdx.x];
-  for (int p = blockIdx.y * FINAL_WARPS + (threadIdx.x >> 5); p < q.P; p += gridDim.y * FINAL_WARPS)
-    finalize_one(q.mode, q.partials, q.flags, q.ychunk, q.P, q.N, q.chunk, q.nchunks, q.fitness, p,
-                 threadIdx.x & 31);
+  const int lanes = merge_lanes(q.nchunks), per = FINAL_THREADS / lanes;
+  const Group g = group_of(lanes);
+  for (int p = blockIdx.y * per + threadIdx.x / lanes; p < q.P; p += gridDim.y * per)
+    finalize_one(q.mode, q.partials, q.flags, q.ychunk, q.P, q.N, q.chunk, q.nchunks, q.fitness, p, g);
 }
 
 // ---------------------------------------------------------------- host side
@@ -1205,27 +1274,23 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
 
   SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.queue, 0, 5 * sizeof(unsigned long long), s));
   if (pl.xform) SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.xneed, 0, (size_t)(xform_rows(nvars, pl.xform) - nvars), s));
-  // one warp per block spreads the serial per-program decode over the SMs
-  st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(decode_kernel));
-  if (st != SR_OK) return st;
   const int stage = pl.stage ? stage_blocks(nvars, N) : 0;
-  decode_kernel<<<(P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
+  const bool centred = mode == MODE_CORR || mode == MODE_BOTH || mode == MODE_R4;
+  double *ych = reinterpret_cast<double *>(ws + pl.off_ych);
+  ep.finite_only = mode == MODE_R4;
+  if (centred) ep.ysum = reinterpret_cast<double *>(ws + pl.off_ysum);
+  const CenterParams cp{y, N, pl.chunk, pl.nchunks, ep.finite_only, ep.ysum, const_cast<float *>(ep.yc), ych};
+  const int yblocks = centred ? pl.nchunks : 0;
+  decode_kernel<<<yblocks + (P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
                   DECODE_WARPS * decode_scratch_bytes(Lmax), s>>>(ep);
   ctx->launches += 1;
   if (pl.xform) {
-    const dim3 g((unsigned)((N + XF_THREADS * 4 - 1) / (XF_THREADS * 4)), (unsigned)xform_rows(nvars, pl.xform));
-    xform_kernel<<<g, XF_THREADS, 0, s>>>(X, ldx, nvars, N, pl.ldxt, ep.xneed,
-                                          reinterpret_cast<float *>(ws + pl.off_xt));
+    xform_kernel<<<yblocks + xform_blocks(nvars, N), XF_THREADS, 0, s>>>(
+        X, ldx, nvars, N, pl.ldxt, pl.xform, ep.xneed, reinterpret_cast<float *>(ws + pl.off_xt), yblocks, cp);
     ctx->launches += 1;
-  }
-  double *ych = reinterpret_cast<double *>(ws + pl.off_ych);
-  if (mode == MODE_CORR || mode == MODE_BOTH || mode == MODE_R4) {
-    double *ysum = reinterpret_cast<double *>(ws + pl.off_ysum);
-    const int r4 = mode == MODE_R4;
-    ysum_kernel<<<pl.nchunks, PREP_THREADS, 0, s>>>(y, N, pl.chunk, r4, ysum);
-    ycenter_kernel<<<pl.nchunks, PREP_THREADS, 0, s>>>(y, N, pl.chunk, pl.nchunks, ysum, r4,
-                                                      const_cast<float *>(ep.yc), ych);
-    ctx->launches += 2;
+  } else if (centred) {
+    ycenter_kernel<<<pl.nchunks, PREP_THREADS, 0, s>>>(cp);
+    ctx->launches += 1;
   }
   if (pl.wide) {
     st = launch_pass(ctx, mode, false, true, pl.minb, pl.smem, ep);
@@ -1245,7 +1310,8 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   if (mode != MODE_PREDICT) {
     FinalParams fp{ep.partials, ep.flags, ych, P, N, pl.chunk, pl.nchunks, mode, fitness, M, counts};
-    finalize_kernel<<<(P + FINAL_WARPS - 1) / FINAL_WARPS, FINAL_WARPS * 32, 0, s>>>(fp);
+    const int per = FINAL_THREADS / merge_lanes(pl.nchunks);
+    finalize_kernel<<<(P + per - 1) / per, FINAL_THREADS, 0, s>>>(fp);
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
   }
@@ -1434,6 +1500,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       bpar->pass = PASS_BASE;
       bpar->decode_blocks = (progs + DECODE_WARPS - 1) / DECODE_WARPS;
       bpar->stage_blocks = stages;
+      bpar->ysum_blocks = corr_chunks;
       bpar->abort = ctx->abort_flag;
       bpar->err = ctx->dev_words;
     }
@@ -1459,29 +1526,25 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
     const size_t g1 = std::min(order.size(), g0 + MAX_BATCH);
     BatchParams b;
     group_bytes(g0, g1, &b);
-    int corr_blocks = 0;
-    for (int r = 0; r < b.ncorr; ++r) corr_blocks += b.prob[b.corr_list[r]].nchunks;
     SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.queue, 0, 5 * sizeof(unsigned long long), s));
     for (int r = 0; r < b.nprob; ++r)
       if (b.prob[r].xform)
         SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.prob[r].xneed, 0,
                                            (size_t)(xform_rows(b.prob[r].nvars, b.prob[r].xform) - b.prob[r].nvars), s));
-    decode_batched_kernel<<<b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
+    decode_batched_kernel<<<b.ysum_blocks + b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
                             DECODE_WARPS * decode_scratch_bytes(maxL), s>>>(b);
     ctx->launches += 1;
     for (size_t g = g0; g < g1; ++g) {  // the variable tables, from the problems' own X
       const BatchProblem &q = b.prob[g - g0];
       if (!q.xform) continue;
       const sr_problem &o = pr[order[g]];
-      const dim3 xg((unsigned)((q.N + XF_THREADS * 4 - 1) / (XF_THREADS * 4)), (unsigned)xform_rows(q.nvars, q.xform));
-      xform_kernel<<<xg, XF_THREADS, 0, s>>>(o.X, o.ldx, q.nvars, q.N, (int)q.ldx, q.xneed,
-                                             const_cast<float *>(q.X));
+      xform_kernel<<<xform_blocks(q.nvars, q.N), XF_THREADS, 0, s>>>(o.X, o.ldx, q.nvars, q.N, (int)q.ldx, q.xform, q.xneed,
+                                                                     const_cast<float *>(q.X), 0, CenterParams{});
       ctx->launches += 1;
     }
     if (b.ncorr > 0) {
-      ysum_batched_kernel<<<corr_blocks, PREP_THREADS, 0, s>>>(b);
-      ycenter_batched_kernel<<<corr_blocks, PREP_THREADS, 0, s>>>(b);
-      ctx->launches += 2;
+      ycenter_batched_kernel<<<b.ysum_blocks, PREP_THREADS, 0, s>>>(b);
+      ctx->launches += 1;
     }
     if (wide) {
       st = launch_batch_pass(ctx, false, true, bminb, smem, b);
@@ -1499,10 +1562,12 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       st = launch_batch_pass(ctx, true, wide, 4, smem_deep, bd);
     }
     if (st != SR_OK) return st;
-    int maxP = 1;
-    for (int r = 0; r < b.nprob; ++r) maxP = b.prob[r].P > maxP ? b.prob[r].P : maxP;
-    const int yblocks = std::min((maxP + FINAL_WARPS - 1) / FINAL_WARPS, 65535);
-    finalize_batched_kernel<<<dim3(b.nprob, yblocks), FINAL_WARPS * 32, 0, s>>>(b);
+    int yblocks = 1;
+    for (int r = 0; r < b.nprob; ++r) {
+      const int per = FINAL_THREADS / merge_lanes(b.prob[r].nchunks);
+      yblocks = std::max(yblocks, std::min((b.prob[r].P + per - 1) / per, 65535));
+    }
+    finalize_batched_kernel<<<dim3(b.nprob, yblocks), FINAL_THREADS, 0, s>>>(b);
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
   }
