@@ -568,7 +568,7 @@ __device__ __noinline__ void accumulate(Acc *acc, V8 T, int c0, int cl, int cl4,
 // Evaluates program `prog` of problem p on case chunk `c` with the calling
 // warp.  MODE_BOTH accumulates the sums selected by `want` (bit 0: squared
 // error, bit 1: correlation moments); the other modes ignore `want`.
-template <int MODE, bool EXT, bool WIDE>
+template <int MODE, bool EXT, bool WIDE, bool LEAN>
 __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, const WarpSmem &w,
                                           int lane, int want) {
   const bool do_mse = MODE == MODE_MSE || (MODE == MODE_BOTH && (want & 1));
@@ -601,7 +601,7 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
     const int c0 = base + CPL * lane;
     const int cl = c0 < cend ? c0 : last_group;           // first 4 cases, always readable
     const int cl4 = cl + 4 < cend ? cl + 4 : cl;          // second 4, or a re-read when none valid
-    const V8 T = interpret<EXT, WIDE, MODE == MODE_P2P>(w.code, stk, p.X + cl, p.X + cl4);
+    const V8 T = interpret<EXT, WIDE, LEAN>(w.code, stk, p.X + cl, p.X + cl4);
     if (MODE == MODE_PREDICT) {
       float tv[CPL];
       unpack8(T, tv);
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_kernel(EvalParams p) {
     const int c = (int)(item / (unsigned long long)p.P);
     const int prog = (int)(item % (unsigned long long)p.P);
     if (!takes(pass, p.ncode[prog])) continue;
-    eval_item<MODE, EXT, WIDE>(p, c, prog, w, lane, 3);
+    eval_item<MODE, EXT, WIDE, MODE == MODE_P2P>(p, c, prog, w, lane, 3);
   }
 }
 
@@ -823,7 +823,13 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const
 // Passes as for eval_kernel.
 // At most 64 registers, so that 4 CTAs fit an SM (75 unbounded, 3 CTAs):
 // 2,608 -> 2,949 GPop/s on the 64-problem batch.
-template <bool EXT, bool WIDE, int MINB>
+// LEAN where items are short: then the code around the interpreter (the item,
+// its problem, the sums) runs as often as its operators and the instruction
+// cache has to hold both.  us with and without, 64 problems of 512 or 1,024
+// programs of <= 64 tokens: 3 steps an item 439 / 562, 6 steps 2,039 / 2,211, 20
+// steps 6,059 / 5,831; 16 problems of <= 128 tokens, 60,000 cases 25,794 / 25,015.
+constexpr int LEAN_MAX_STEPS = 10;
+template <bool EXT, bool WIDE, int MINB, bool LEAN>
 __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int pass = EXT ? b.pass : PASS_BASE;
@@ -847,7 +853,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __
     const int prog = (int)(local % q.P);
     if (!takes(pass, q.ncode[prog])) continue;
     const int want = q.mode == MODE_MSE ? 1 : (q.mode == MODE_CORR ? 2 : 3);
-    eval_item<MODE_BOTH, EXT, WIDE>(p, c, prog, w, lane, want);
+    eval_item<MODE_BOTH, EXT, WIDE, LEAN>(p, c, prog, w, lane, want);
   }
 }
 
@@ -1320,14 +1326,17 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
 
 // ---------------------------------------------------------------- batched host side
 typedef void (*BatchKernel)(const BatchParams);
-BatchKernel batch_kernel_for(bool ext, bool wide, int minb) {
-  if (!wide) return eval_batched_kernel<true, false, 4>;
-  if (minb == 3) return ext ? eval_batched_kernel<true, true, 3> : eval_batched_kernel<false, true, 3>;
-  if (minb == 5) return ext ? eval_batched_kernel<true, true, 5> : eval_batched_kernel<false, true, 5>;
-  return ext ? eval_batched_kernel<true, true, 4> : eval_batched_kernel<false, true, 4>;
+template <int MINB>
+BatchKernel batch_kernel_m(bool ext, bool lean) {
+  if (ext) return eval_batched_kernel<true, true, MINB, false>;
+  return lean ? eval_batched_kernel<false, true, MINB, true> : eval_batched_kernel<false, true, MINB, false>;
 }
-sr_status launch_batch_pass(sr_ctx *ctx, bool ext, bool wide, int minb, int smem, const BatchParams &b) {
-  const BatchKernel k = batch_kernel_for(ext, wide, minb);
+BatchKernel batch_kernel_for(bool ext, bool wide, int minb, bool lean) {
+  if (!wide) return eval_batched_kernel<true, false, 4, false>;
+  return minb == 3 ? batch_kernel_m<3>(ext, lean) : (minb == 5 ? batch_kernel_m<5>(ext, lean) : batch_kernel_m<4>(ext, lean));
+}
+sr_status launch_batch_pass(sr_ctx *ctx, bool ext, bool wide, int minb, int smem, const BatchParams &b, bool lean = false) {
+  const BatchKernel k = batch_kernel_for(ext, wide, minb, lean);
   int grid = 0;
   sr_status st = persistent_grid(ctx, reinterpret_cast<const void *>(k), smem, &grid);
   if (st != SR_OK) return st;
@@ -1547,7 +1556,9 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       ctx->launches += 1;
     }
     if (wide) {
-      st = launch_batch_pass(ctx, false, true, bminb, smem, b);
+      double steps = 0.0;
+      for (int r = 0; r < b.nprob; ++r) steps += (double)b.prob[r].P * ((b.prob[r].N + STEP - 1) / STEP);
+      st = launch_batch_pass(ctx, false, true, bminb, smem, b, steps <= (double)LEAN_MAX_STEPS * (double)b.total_items);
       b.pass = PASS_EXT;
       if (st == SR_OK) st = launch_batch_pass(ctx, true, true, bminb, smem, b);
     } else {

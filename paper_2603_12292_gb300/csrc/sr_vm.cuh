@@ -296,7 +296,7 @@ struct Shape {
 // EXT: the copy that also runs 1/x, tan, asin, acos, atan, tanh.
 // WIDE: rows start on 32-byte boundaries and hold whole groups of 8 cases (one
 // 256-bit load a row); else two 128-bit loads.
-// LEAN: the kernel around it is large (Shape).
+// LEAN: the code around it is large, or runs nearly as often (Shape).
 template <bool EXT, bool WIDE, bool LEAN>
 __device__ __forceinline__ V8 interpret(const uint2 *code, const char *stk, const float *__restrict__ xa,
                                         const float *__restrict__ xb) {

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2603_12292_gb300 import binding
+from paper_2603_12292_gb300 import binding, inputs
 from progtext import pack, parse
 
 pytestmark = pytest.mark.gpu
@@ -43,3 +43,25 @@ def test_fitness_for_any_number_of_chunks(ctx, chunks):
         assert abs(got[0, p] - mse) <= 2.0 ** -20 * mse, (text, p)
         want = 1.0 if text == "c0" else 1.0 - np.corrcoef(out[p], y64)[0, 1] ** 2
         assert abs(got[1, p] - want) <= 2.0 ** -17, (text, p)
+
+
+@pytest.mark.parametrize("tile", [256, 2560, 2816, 6144])
+def test_batched_items_short_and_long_equal_single_calls(ctx, tile):
+    """Both copies of the batched kernel (short and long items) against sr_eval with the same chunks."""
+    rng = np.random.default_rng(tile)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    probs, single = [], []
+    binding.sr_set_tile(ctx, tile)
+    try:
+        for i, N in enumerate((6144, 6001, 12_288)):
+            pr = inputs.make_problem("items", 70 + i, P=90, Lmin=1, Lmax=40, nvars=3, K=2, N=N, xlo=-2.0, xhi=2.0,
+                                     target_len=(3, 7), unary_ops=12 if i == 1 else 6)
+            y = t(rng.normal(0, 1, N).astype(np.float32))
+            args = (t(pr.programs), t(pr.lengths), t(pr.consts), t(pr.X), y, N, binding.SR_MSE_CORR)
+            single.append(binding.sr_eval(ctx, *args))
+            probs.append(binding.make_problem(*args, cases_per_tile=tile))
+        got = binding.sr_eval_batched(ctx, probs)
+    finally:
+        binding.sr_set_tile(ctx, 0)
+    for a, b in zip(got, single):
+        assert torch.equal(a, b)
