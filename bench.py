@@ -37,8 +37,8 @@ CSRC = os.path.join(ROOT, "paper_2603_12292_gb300", "csrc")
 # The CUDA sources each dominant kernel is built from: an ncu figure below is
 # reported only while these files hash to what they were when it was captured.
 KERNEL_SOURCES = {
-    "eval": ("sr_eval.cu", "sr_interp.cuh", "sr_common.cuh"),
-    "grad": ("sr_grad.cu", "sr_interp.cuh", "sr_common.cuh"),
+    "eval": ("sr_eval.cu", "sr_vm.cuh", "sr_decode.cuh", "sr_interp.cuh", "sr_common.cuh"),
+    "grad": ("sr_grad.cu", "sr_gradvm.cuh", "sr_vm.cuh", "sr_decode.cuh", "sr_interp.cuh", "sr_common.cuh"),
 }
 # Dominant kernels of the workloads, each from one ncu --set full capture
 # summarised under profiles/: the captured workload, DRAM bytes (read +

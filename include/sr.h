@@ -437,12 +437,13 @@ sr_status sr_random_programs(sr_ctx *ctx, uint8_t *prog, int32_t *len, float *c,
 /*
  * sr_eval_grad -- MSE of every program and its gradient with respect to the
  * program's constants: dconst[p][k] = (2/N) sum_i (yhat_i - y_i) dyhat_i/dc_k.
- * Per (program, case) the forward pass is recomputed into an on-chip tape
- * (one value per token, shared memory) and swept in reverse with an adjoint
- * stack.  Derivative conventions: a protected fallback branch, a clamped exp
- * and sqrt|x| at x = 0 have derivative 0; d log|x|/dx = 1/x; d sqrt|x|/dx =
- * sign(x) / (2 sqrt|x|).  FP32 per case, FP32 compensated sums per lane,
- * FP64 across lanes and case chunks.
+ * Per (program, case) the forward pass is recomputed onto a tape (what the
+ * reverse pass needs and cannot have as a constant or a row of X) and swept in
+ * reverse; subtrees that read only constants are evaluated once.  Derivative
+ * conventions: a protected fallback branch, a clamped exp and sqrt|x| at x = 0
+ * have derivative 0; d log|x|/dx = 1/x; d sqrt|x|/dx = sign(x) / (2 sqrt|x|).
+ * FP32 per case, FP32 compensated sums per lane, FP64 across lanes and case
+ * chunks.
  *   arguments as sr_eval; mse device double [P]; dconst device double
  *   [P][K] (K >= 1).  Invalid programs: mse = +inf, dconst = 0.
  * Errors: SR_EINVAL, SR_ENOMEM, SR_ECUDA.

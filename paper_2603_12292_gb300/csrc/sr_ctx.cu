@@ -3,6 +3,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -23,6 +24,11 @@ sr_status fail(sr_ctx *ctx, sr_status s, const char *fmt, ...) {
 
 sr_status cuda_fail(sr_ctx *ctx, cudaError_t e, const char *what) {
   return fail(ctx, SR_ECUDA, "%s: %s", what, cudaGetErrorString(e));
+}
+
+unsigned long long call_tag() {
+  static std::atomic<unsigned long long> calls{0};
+  return ++calls;
 }
 
 bool stream_capturing(sr_ctx *ctx) {

@@ -8,14 +8,13 @@
 // Eq. 1, scored here as 1 - r^2 (Sec. 2.1.5).
 //
 // Design on the device
-//   1. Decode pre-pass, a warp per program (lane 0 walks the tree in shared
-//      memory): validation, then the expression tree is rescheduled
-//      Sethi-Ullman style -- at every binary node the child that needs more
-//      stack is evaluated first (a reversed opcode keeps a - b and a / b
-//      exact when the right child goes first).  The stack depth of any
-//      program is then at most floor(log2(leaves)) + 1 (9 for 512 tokens), so
-//      floor(log2((Lmax + 1) / 2)) slots always suffice; most programs need
-//      far fewer, so the main passes give each warp only what fits 4 or 5
+//   1. Decode pre-pass, a warp per program (sr_decode.cuh): validation, then the
+//      expression tree is rescheduled Sethi-Ullman style -- at every binary node
+//      the child that needs more stack is evaluated first (a reversed opcode
+//      keeps a - b and a / b exact when the right child goes first).  The stack
+//      depth of any program is then at most floor(log2(leaves)) + 1 (9 for 512
+//      tokens), so floor(log2((Lmax + 1) / 2)) slots always suffice; most programs
+//      need far fewer, so the main passes give each warp only what fits 4 or 5
 //      CTAs per SM and the rare deeper programs run in a third pass.
 //      A terminal evaluated second is fused into its binary operator
 //      ("top = top op x_j"), and every operand is resolved here (constant
@@ -26,13 +25,15 @@
 //      handed out chunk-major by one atomic counter to single warps, so
 //      warps running together share X columns in L1/L2 and uneven program
 //      lengths balance out.  The warp copies the program's code into shared
-//      memory and interprets it with lanes over cases, 8 cases per lane (two
-//      float4 per operand), 256 cases per step; the op stream is
-//      warp-uniform (no divergence).  Top of stack in registers, the slots
-//      below in shared memory [slot][half][lane] (conflict-free float4).
-//   3. Per lane, FP32 Kahan-compensated sums over the item's cases; FP64 warp
+//      memory and interprets it with lanes over cases, 8 cases per lane, 256
+//      cases per step (sr_vm.cuh); the op stream is warp-uniform (no
+//      divergence).  Top of stack in registers, the slots below in shared
+//      memory [slot][half][lane] (conflict-free float4).
+//   3. Per lane, FP32 Kahan-compensated sums over the item's cases, out of line
+//      and in local memory, so that they cost the interpreter no registers
+//      (4,096 x 100,000 at 5 CTAs per SM: 5,824 -> 5,434 us); FP64 warp
 //      reduction; one FP64 partial per (program, chunk); a finalize kernel
-//      merges the chunks of each program (a warp per program, fixed order).
+//      merges the chunks of each program (a group of lanes each, fixed order).
 #include <math.h>
 #include <stdio.h>
 
@@ -93,9 +94,11 @@ struct EvalParams {
   int32_t *flags;          // [P]
   uint2 *code;             // [P][Lmax] decoded instructions
   int32_t *ncode;          // [P]
-  // [0] work counter, [1] work counter of the EXT pass, [2] EXT programs,
-  // [3] work counter of the deep pass, [4] deep programs
+  // [0] work counter, [1] work counter of the EXT pass, [2] `tag` when it has
+  // programs, [3], [4] the same of the deep pass; the decode launch zeroes the
+  // counters and notes the tags
   unsigned long long *queue;
+  unsigned long long tag;  // call_tag
   float *yhat;             // predict: [P][ldy]
   long long ldy;
   int warp_bytes;          // shared memory per warp
@@ -257,9 +260,8 @@ __device__ void ycenter_chunk(const float *__restrict__ y, int N, int chunk, int
 
 
 // ---------------------------------------------------------------- decode pre-pass
-// cap_slots: programs that need more get NCODE_DEEP, counted in deep_count
-__device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_slots,
-                                                  unsigned long long *deep_count) {
+// cap_slots: programs that need more get NCODE_DEEP
+__device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_slots) {
   DecodeArgs a;
   a.programs = p.programs;
   a.lengths = p.lengths;
@@ -272,10 +274,11 @@ __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_s
   a.code = p.code;
   a.ncode = p.ncode;
   a.flags = p.flags;
-  a.ext_count = p.queue ? p.queue + 2 : nullptr;
   a.max_slots = slots_for(p.Lmax);
   a.cap_slots = cap_slots;
-  a.deep_count = deep_count;
+  a.ext_note = p.queue + 2;
+  a.deep_note = p.queue + 4;
+  a.tag = p.tag;
   a.xform = p.xform;
   a.xneed = p.xneed;
   return a;
@@ -301,6 +304,8 @@ __device__ void stage_rows(const EvalParams &p, int block) {
 __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ double red[DECODE_WARPS];
+  launch_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.queue[0] = p.queue[1] = p.queue[3] = 0;
   const int yblocks = p.ysum ? p.nchunks : 0, dblocks = (p.P + DECODE_WARPS - 1) / DECODE_WARPS;
   const int block = (int)blockIdx.x - yblocks;
   if (block < 0) {
@@ -313,7 +318,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_kernel(EvalParams p)
   }
   const int warp = threadIdx.x >> 5, prog = block * DECODE_WARPS + warp;
   if (prog < p.P)
-    decode_eval_warp(decode_args(p, p.slots, p.queue + 4), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
+    decode_eval_warp(decode_args(p, p.slots), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
 }
 
 // The variable table of an evaluation with transforms (DecodeArgs::xform):
@@ -374,6 +379,7 @@ struct CenterParams {
 };
 __global__ void __launch_bounds__(PREP_THREADS) ycenter_kernel(CenterParams y) {
   __shared__ double red[PREP_THREADS / 32];
+  launch_wait();
   ycenter_chunk(y.y, y.N, y.chunk, y.nchunks, blockIdx.x, y.ysum, y.nan_invalid != 0, y.yc, y.ychunk, red);
 }
 // The first yblocks blocks centre the target, one chunk each.
@@ -381,6 +387,7 @@ __global__ void __launch_bounds__(XF_THREADS)
     xform_kernel(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt, int depth,
                  const uint8_t *__restrict__ xneed, float *__restrict__ xt, int yblocks, CenterParams y) {
   __shared__ double red[XF_THREADS / 32];
+  launch_wait();
   const int block = (int)blockIdx.x - yblocks, per_part = (N + XF_THREADS * 4 - 1) / (XF_THREADS * 4);
   if (block < 0) {
     ycenter_chunk(y.y, y.N, y.chunk, y.nchunks, blockIdx.x, y.ysum, y.nan_invalid != 0, y.yc, y.ychunk, red);
@@ -662,7 +669,7 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
 // ---------------------------------------------------------------- single problem
 // Up to three passes over the work items: the programs of the base operators
 // (and the invalid ones), those that use 1/x, tan, asin, acos, atan or tanh
-// (which returns at once when the decoder counted none), and those that need
+// (which returns at once when there are none), and those that need
 // more than the main passes' shallow_slots(Lmax, MINB) stack slots (NCODE_DEEP;
 // made only when slots_for(Lmax) is more).  Keeping the extended operators out
 // of the first kernel keeps its loop inside the instruction cache.  Where the
@@ -676,17 +683,18 @@ __device__ __forceinline__ bool takes(int pass, int ncode) {
   return pass == PASS_SHALLOW || ncode_ext(ncode) == (pass == PASS_EXT);
 }
 // the pass's work counter; NULL when it has no programs
-__device__ __forceinline__ unsigned long long *pass_queue(unsigned long long *queue, int pass) {
-  if (pass == PASS_EXT) return queue[2] ? queue + 1 : nullptr;
-  if (pass == PASS_DEEP) return queue[4] ? queue + 3 : nullptr;
+__device__ __forceinline__ unsigned long long *pass_queue(unsigned long long *queue, int pass, unsigned long long tag) {
+  if (pass == PASS_EXT) return queue[2] == tag ? queue + 1 : nullptr;
+  if (pass == PASS_DEEP) return queue[4] == tag ? queue + 3 : nullptr;
   return queue;
 }
 
 template <int MODE, bool EXT, bool WIDE, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB) eval_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
+  launch_wait();
   const int pass = EXT ? p.pass : PASS_BASE;
-  unsigned long long *q = pass_queue(p.queue, pass);
+  unsigned long long *q = pass_queue(p.queue, pass, p.tag);
   if (!q) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, p.warp_bytes, p.slots);
@@ -738,6 +746,7 @@ struct BatchParams {
   int total_progs;
   long long total_items;
   unsigned long long *queue;  // as EvalParams::queue
+  unsigned long long tag;
   int warp_bytes;
   int slots;
   int maxL;                   // the largest Lmax of the batch
@@ -789,6 +798,8 @@ __device__ __forceinline__ int corr_problem_of_block(const BatchParams &b) {
 __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char dsm[];
   __shared__ double red[DECODE_WARPS];
+  launch_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) b.queue[0] = b.queue[1] = b.queue[3] = 0;
   const int block = (int)blockIdx.x - b.ysum_blocks;
   if (block < 0) {
     const BatchProblem &q = b.prob[corr_problem_of_block(b)];
@@ -814,7 +825,8 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const
   }
   EvalParams p = view(b.prob[lo]);
   p.queue = b.queue;
-  decode_eval_warp(decode_args(p, b.slots, b.queue + 4), g - b.prob[lo].prog_begin,
+  p.tag = b.tag;
+  decode_eval_warp(decode_args(p, b.slots), g - b.prob[lo].prog_begin,
                    dsm + (size_t)warp * decode_scratch_bytes(b.maxL));
 }
 
@@ -832,8 +844,9 @@ constexpr int LEAN_MAX_STEPS = 10;
 template <bool EXT, bool WIDE, int MINB, bool LEAN>
 __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __grid_constant__ BatchParams b) {
   extern __shared__ __align__(16) unsigned char smem[];
+  launch_wait();
   const int pass = EXT ? b.pass : PASS_BASE;
-  unsigned long long *qc = pass_queue(b.queue, pass);
+  unsigned long long *qc = pass_queue(b.queue, pass, b.tag);
   if (!qc) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, b.warp_bytes, b.slots);
@@ -1040,6 +1053,7 @@ struct FinalParams {
 constexpr int FINAL_THREADS = 128;
 
 __global__ void __launch_bounds__(FINAL_THREADS) finalize_kernel(FinalParams f) {
+  launch_wait();
   const int lanes = merge_lanes(f.nchunks), p = (blockIdx.x * FINAL_THREADS + threadIdx.x) / lanes;
   if (p >= f.P) return;
   finalize_one(f.mode, f.partials, f.flags, f.ychunk, f.P, f.N, f.chunk, f.nchunks, f.fitness, p, group_of(lanes), f.M,
@@ -1052,6 +1066,7 @@ __global__ void __launch_bounds__(FINAL_THREADS) finalize_kernel(FinalParams f) 
 
 __global__ void __launch_bounds__(PREP_THREADS) ycenter_batched_kernel(const __grid_constant__ BatchParams b) {
   __shared__ double red[PREP_THREADS / 32];
+  launch_wait();
   const BatchProblem &q = b.prob[corr_problem_of_block(b)];
   ycenter_chunk(q.y, q.N, q.chunk, q.nchunks, (int)blockIdx.x - q.corr_chunk_begin, q.ysum, false, q.yc,
                 q.ychunk, red);
@@ -1059,6 +1074,7 @@ __global__ void __launch_bounds__(PREP_THREADS) ycenter_batched_kernel(const __g
 
 // blocks (problem, FINAL_THREADS / merge_lanes programs of it)
 __global__ void __launch_bounds__(FINAL_THREADS) finalize_batched_kernel(const __grid_constant__ BatchParams b) {
+  launch_wait();
   const BatchProblem &q = b.prob[blockIdx.x];
   const int lanes = merge_lanes(q.nchunks), per = FINAL_THREADS / lanes;
   const Group g = group_of(lanes);
@@ -1105,7 +1121,7 @@ sr_status launch_pass(sr_ctx *ctx, int mode, bool ext, bool wide, int minb, int 
   int grid = 0;
   sr_status st = persistent_grid(ctx, reinterpret_cast<const void *>(k), smem, &grid);
   if (st != SR_OK) return st;
-  k<<<grid, WARPS * 32, smem, ctx->stream>>>(ep);
+  SR_CHECK_CUDA(ctx, launch(k, grid, WARPS * 32, smem, ctx->stream, ep));
   ctx->launches += 1;
   return SR_OK;
 }
@@ -1259,6 +1275,7 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   ep.code = reinterpret_cast<uint2 *>(ws + pl.off_code);
   ep.ncode = reinterpret_cast<int32_t *>(ws + pl.off_ncode);
   ep.queue = reinterpret_cast<unsigned long long *>(ws + pl.off_queue);
+  ep.tag = call_tag();
   ep.yhat = yhat;
   ep.ldy = ldy;
   ep.slots = pl.slots;
@@ -1278,7 +1295,6 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
     ep.ldsrc = ldx;
   }
 
-  SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.queue, 0, 5 * sizeof(unsigned long long), s));
   if (pl.xform) SR_CHECK_CUDA(ctx, cudaMemsetAsync(ep.xneed, 0, (size_t)(xform_rows(nvars, pl.xform) - nvars), s));
   const int stage = pl.stage ? stage_blocks(nvars, N) : 0;
   const bool centred = mode == MODE_CORR || mode == MODE_BOTH || mode == MODE_R4;
@@ -1287,15 +1303,15 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   if (centred) ep.ysum = reinterpret_cast<double *>(ws + pl.off_ysum);
   const CenterParams cp{y, N, pl.chunk, pl.nchunks, ep.finite_only, ep.ysum, const_cast<float *>(ep.yc), ych};
   const int yblocks = centred ? pl.nchunks : 0;
-  decode_kernel<<<yblocks + (P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
-                  DECODE_WARPS * decode_scratch_bytes(Lmax), s>>>(ep);
+  SR_CHECK_CUDA(ctx, launch(decode_kernel, yblocks + (P + DECODE_WARPS - 1) / DECODE_WARPS + stage, DECODE_WARPS * 32,
+                            DECODE_WARPS * decode_scratch_bytes(Lmax), s, ep));
   ctx->launches += 1;
   if (pl.xform) {
-    xform_kernel<<<yblocks + xform_blocks(nvars, N), XF_THREADS, 0, s>>>(
-        X, ldx, nvars, N, pl.ldxt, pl.xform, ep.xneed, reinterpret_cast<float *>(ws + pl.off_xt), yblocks, cp);
+    SR_CHECK_CUDA(ctx, launch(xform_kernel, yblocks + xform_blocks(nvars, N), XF_THREADS, 0, s, X, ldx, nvars, N, pl.ldxt,
+                              pl.xform, ep.xneed, reinterpret_cast<float *>(ws + pl.off_xt), yblocks, cp));
     ctx->launches += 1;
   } else if (centred) {
-    ycenter_kernel<<<pl.nchunks, PREP_THREADS, 0, s>>>(cp);
+    SR_CHECK_CUDA(ctx, launch(ycenter_kernel, pl.nchunks, PREP_THREADS, 0, s, cp));
     ctx->launches += 1;
   }
   if (pl.wide) {
@@ -1317,7 +1333,7 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   if (mode != MODE_PREDICT) {
     FinalParams fp{ep.partials, ep.flags, ych, P, N, pl.chunk, pl.nchunks, mode, fitness, M, counts};
     const int per = FINAL_THREADS / merge_lanes(pl.nchunks);
-    finalize_kernel<<<(P + per - 1) / per, FINAL_THREADS, 0, s>>>(fp);
+    SR_CHECK_CUDA(ctx, launch(finalize_kernel, (P + per - 1) / per, FINAL_THREADS, 0, s, fp));
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
   }
@@ -1340,7 +1356,7 @@ sr_status launch_batch_pass(sr_ctx *ctx, bool ext, bool wide, int minb, int smem
   int grid = 0;
   sr_status st = persistent_grid(ctx, reinterpret_cast<const void *>(k), smem, &grid);
   if (st != SR_OK) return st;
-  k<<<grid, WARPS * 32, smem, ctx->stream>>>(b);
+  SR_CHECK_CUDA(ctx, launch(k, grid, WARPS * 32, smem, ctx->stream, b));
   ctx->launches += 1;
   return SR_OK;
 }
@@ -1535,24 +1551,24 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
     const size_t g1 = std::min(order.size(), g0 + MAX_BATCH);
     BatchParams b;
     group_bytes(g0, g1, &b);
-    SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.queue, 0, 5 * sizeof(unsigned long long), s));
+    b.tag = call_tag();
     for (int r = 0; r < b.nprob; ++r)
       if (b.prob[r].xform)
         SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.prob[r].xneed, 0,
                                            (size_t)(xform_rows(b.prob[r].nvars, b.prob[r].xform) - b.prob[r].nvars), s));
-    decode_batched_kernel<<<b.ysum_blocks + b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
-                            DECODE_WARPS * decode_scratch_bytes(maxL), s>>>(b);
+    SR_CHECK_CUDA(ctx, launch(decode_batched_kernel, b.ysum_blocks + b.decode_blocks + b.stage_blocks, DECODE_WARPS * 32,
+                              DECODE_WARPS * decode_scratch_bytes(maxL), s, b));
     ctx->launches += 1;
     for (size_t g = g0; g < g1; ++g) {  // the variable tables, from the problems' own X
       const BatchProblem &q = b.prob[g - g0];
       if (!q.xform) continue;
       const sr_problem &o = pr[order[g]];
-      xform_kernel<<<xform_blocks(q.nvars, q.N), XF_THREADS, 0, s>>>(o.X, o.ldx, q.nvars, q.N, (int)q.ldx, q.xform, q.xneed,
-                                                                     const_cast<float *>(q.X), 0, CenterParams{});
+      SR_CHECK_CUDA(ctx, launch(xform_kernel, xform_blocks(q.nvars, q.N), XF_THREADS, 0, s, o.X, o.ldx, q.nvars, q.N, (int)q.ldx,
+                                q.xform, q.xneed, const_cast<float *>(q.X), 0, CenterParams{}));
       ctx->launches += 1;
     }
     if (b.ncorr > 0) {
-      ycenter_batched_kernel<<<b.ysum_blocks, PREP_THREADS, 0, s>>>(b);
+      SR_CHECK_CUDA(ctx, launch(ycenter_batched_kernel, b.ysum_blocks, PREP_THREADS, 0, s, b));
       ctx->launches += 1;
     }
     if (wide) {
@@ -1578,7 +1594,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       const int per = FINAL_THREADS / merge_lanes(b.prob[r].nchunks);
       yblocks = std::max(yblocks, std::min((b.prob[r].P + per - 1) / per, 65535));
     }
-    finalize_batched_kernel<<<dim3(b.nprob, yblocks), FINAL_THREADS, 0, s>>>(b);
+    SR_CHECK_CUDA(ctx, launch(finalize_batched_kernel, dim3(b.nprob, yblocks), FINAL_THREADS, 0, s, b));
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
   }

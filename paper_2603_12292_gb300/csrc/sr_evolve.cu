@@ -124,6 +124,7 @@ __global__ void tournament_kernel(const double *__restrict__ fitness, int P, int
                                   int32_t *__restrict__ parents) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * P) return;
+  launch_wait();
   const Rng rng = rng_in.resolved();
   const int i = t >> 1, s = t & 1;
   int best = 0x7fffffff;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * VARY_WARPS + warp;
   if (i >= p.P) return;
+  launch_wait();
   // out-of-range parents and lengths are clamped so that no access leaves
   // the buffers (valid inputs are unaffected)
   const int ia = min(max(p.parents[2 * i], 0), p.P_in - 1);
@@ -471,9 +473,9 @@ static sr_status select_tournament(sr_ctx *ctx, const double *fitness, int P, in
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
   const Rng rng = make_rng(seed, gen, ctx->gen_dev);
   if (maximise)
-    tournament_kernel<1><<<(2 * P + 255) / 256, 256, 0, ctx->stream>>>(fitness, P, k, rng, parents);
+    SR_CHECK_CUDA(ctx, launch(tournament_kernel<1>, (2 * P + 255) / 256, 256, 0, ctx->stream, fitness, P, k, rng, parents));
   else
-    tournament_kernel<0><<<(2 * P + 255) / 256, 256, 0, ctx->stream>>>(fitness, P, k, rng, parents);
+    SR_CHECK_CUDA(ctx, launch(tournament_kernel<0>, (2 * P + 255) / 256, 256, 0, ctx->stream, fitness, P, k, rng, parents));
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   ctx->launches += 1;
   return SR_OK;
@@ -506,8 +508,8 @@ sr_status sr_vary(sr_ctx *ctx, const uint8_t *prog_in, const int32_t *len_in, co
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
   VaryParams vp{prog_in, len_in, c_in, parents, prog_out, len_out, c_out, P, Lmax, K, nvars, *cfg,
                 make_rng(seed, gen, ctx->gen_dev), P_in};
-  vary_kernel<<<(P + VARY_WARPS - 1) / VARY_WARPS, VARY_WARPS * 32, VARY_WARPS * 3 * vary_row_bytes(Lmax),
-                ctx->stream>>>(vp);
+  SR_CHECK_CUDA(ctx, launch(vary_kernel, (P + VARY_WARPS - 1) / VARY_WARPS, VARY_WARPS * 32,
+                            VARY_WARPS * 3 * vary_row_bytes(Lmax), ctx->stream, vp));
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   ctx->launches += 1;
   return SR_OK;

