@@ -164,15 +164,23 @@ struct VaryParams {
   int P_in;  // parents' population size
 };
 
-// One warp per child, every step by the whole warp: both parents' rows come
-// into shared memory with the widest loads their stride allows, a subtree's
-// first token is found from prefix sums of the stack effects (two ballots give
-// 32 of them), the child is gathered four bytes a lane, lane k holds constant
-// k, and the five Philox draws of a child run on five lanes at once.  What
-// bounds it: issue slots, then the latency of the rows' gather.  262,144
-// children of <= 256 tokens, K = 4: 631 us with lane 0 walking the rows byte by
-// byte, 2,280 warp instructions a child; now 174 us and 618.
-constexpr int VARY_WARPS = 4;
+// A group of G lanes (a warp or half of one) per child, every step by the whole
+// group: both parents' rows come into shared memory with the widest loads their
+// stride allows, a subtree's first token is found from prefix sums of the stack
+// effects (two ballots give G of them), the child is gathered four bytes a lane,
+// lane k holds constant k, and the five Philox draws of a child run on five lanes
+// at once.  What bounds it: issue slots, then the latency of the rows' gather.
+// 262,144 children of <= 256 tokens, K = 4: 631 us with lane 0 of a warp walking
+// the rows byte by byte, 2,280 warp instructions a child; by the whole warp 174 us
+// and 618; by half a warp each 165 us.
+// Half a warp per child where there are enough children to fill the GPU so: what
+// a child costs whatever its length is shared by two, and long rows take twice the
+// rounds.  A warp, half a warp per child: 8,192 children of <= 64 tokens 8.5, 8.2 us,
+// 65,536 of them 40.9, 32.4; 16,384 of <= 256 tokens 15.0, 16.1, 32,768 of them 25.9,
+// 25.3, 262,144 of them 181.9, 164.9; 1,024 of <= 64 tokens 4.9, 6.2.
+constexpr int VARY_THREADS = 128;
+inline bool vary_halves(int P, int Lmax) { return P >= 8192 && P >= 128 * Lmax; }
+static_assert(SR_MAX_CONSTS <= 16, "a lane of the group holds one constant of the child");
 __host__ __device__ inline int vary_row_bytes(int Lmax) { return (Lmax + 15) & ~15; }
 
 // bytes per load or store of a row: rows of Lmax bytes from base
@@ -181,27 +189,46 @@ __device__ __forceinline__ int row_grain(const uint8_t *base, int Lmax) {
   return (m & 15) == 0 ? 16 : ((m & 3) == 0 ? 4 : 1);
 }
 // the first n bytes (or a few more of the row) of a global row into shared memory
+template <int G>
 __device__ __forceinline__ void load_row(uint8_t *dst, const uint8_t *src, int n, int grain, int lane) {
   if (grain == 16) {
-    if (lane * 16 < n) reinterpret_cast<uint4 *>(dst)[lane] = __ldg(reinterpret_cast<const uint4 *>(src) + lane);
+    for (int t = lane; t * 16 < n; t += G)
+      reinterpret_cast<uint4 *>(dst)[t] = __ldg(reinterpret_cast<const uint4 *>(src) + t);
   } else if (grain == 4) {
-    for (int t = lane; t * 4 < n; t += 32)
+    for (int t = lane; t * 4 < n; t += G)
       reinterpret_cast<uint32_t *>(dst)[t] = __ldg(reinterpret_cast<const uint32_t *>(src) + t);
   } else {
-    for (int t = lane; t < n; t += 32) dst[t] = __ldg(src + t);
+    for (int t = lane; t < n; t += G) dst[t] = __ldg(src + t);
   }
 }
 
-// First token of the subtree whose root is `end`, by the warp: the largest t <= end with the stack effects of
+// Lanes of a group: its bits in a warp's masks, and votes within it.
+template <int G>
+struct Lanes {
+  unsigned mask;
+  int shift, lane;
+  __device__ __forceinline__ Lanes() {
+    const int l = threadIdx.x & 31;
+    lane = l & (G - 1);
+    shift = l & ~(G - 1);
+    mask = (G == 32 ? FULL : (1u << (G & 31)) - 1u) << shift;
+  }
+  __device__ __forceinline__ unsigned ballot(bool b) const { return (__ballot_sync(mask, b) & mask) >> shift; }
+  __device__ __forceinline__ uint32_t get(uint32_t v, int from) const { return __shfl_sync(mask, v, from, G); }
+  __device__ __forceinline__ void sync() const { __syncwarp(mask); }
+};
+
+// First token of the subtree whose root is `end`, by the group: the largest t <= end with the stack effects of
 // tok[t .. end] summing to 1, or 0 if there is none
-__device__ __forceinline__ int warp_subtree_start(const uint8_t *tok, int end, int lane) {
-  const unsigned upto = 0xffffffffu >> (31 - lane);  // lanes 0 .. lane
+template <int G>
+__device__ __forceinline__ int group_subtree_start(const Lanes<G> &g, const uint8_t *tok, int end) {
+  const unsigned upto = 0xffffffffu >> (31 - g.lane);  // lanes 0 .. lane
   int acc = 0;
-  for (int top = end; top >= 0; top -= 32) {
-    const int t = top - lane;
+  for (int top = end; top >= 0; top -= G) {
+    const int t = top - g.lane;
     const int e = t >= 0 ? effect(tok[t]) : 0;
-    const unsigned up = __ballot_sync(FULL, e > 0), down = __ballot_sync(FULL, e < 0);
-    const unsigned hit = __ballot_sync(FULL, t >= 0 && acc + __popc(up & upto) - __popc(down & upto) == 1);
+    const unsigned up = g.ballot(e > 0), down = g.ballot(e < 0);
+    const unsigned hit = g.ballot(t >= 0 && acc + __popc(up & upto) - __popc(down & upto) == 1);
     if (hit) return top - (__ffs(hit) - 1);
     acc += __popc(up) - __popc(down);
   }
@@ -216,10 +243,12 @@ __device__ __forceinline__ uint32_t const_bit(uint32_t v) {
   return r;
 }
 
-__global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
+template <int G>
+__global__ void __launch_bounds__(VARY_THREADS) vary_kernel(VaryParams p) {
   extern __shared__ __align__(16) uint8_t vsm[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * VARY_WARPS + warp;
+  const Lanes<G> g;
+  const int lane = g.lane, group = threadIdx.x / G;
+  const int i = blockIdx.x * (VARY_THREADS / G) + group;
   if (i >= p.P) return;
   launch_wait();
   // out-of-range parents and lengths are clamped so that no access leaves
@@ -228,10 +257,10 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   const int ib = min(max(p.parents[2 * i + 1], 0), p.P_in - 1);
   const int la = min(max(p.len_in[ia], 1), p.Lmax), lb = min(max(p.len_in[ib], 1), p.Lmax);
   const int R = vary_row_bytes(p.Lmax);
-  uint8_t *sA = vsm + (size_t)warp * 3 * R, *sB = sA + R, *out = sB + R;
+  uint8_t *sA = vsm + (size_t)group * 3 * R, *sB = sA + R, *out = sB + R;
   const int grain = row_grain(p.prog_in, p.Lmax);
-  load_row(sA, p.prog_in + (size_t)ia * p.Lmax, la, grain, lane);
-  load_row(sB, p.prog_in + (size_t)ib * p.Lmax, lb, grain, lane);
+  load_row<G>(sA, p.prog_in + (size_t)ia * p.Lmax, la, grain, lane);
+  load_row<G>(sB, p.prog_in + (size_t)ib * p.Lmax, lb, grain, lane);
   float c = 0.0f, cb = 0.0f;  // constant `lane` of the child, and of parent B
   if (lane < p.K) {
     c = p.c_in[(size_t)ia * p.K + lane];
@@ -240,10 +269,10 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   // draw 0 of the decisions and of every kind of variation, one per lane
   const Rng rng = p.rng.resolved();
   const Word4 w = rng.draw(0, (uint32_t)i, lane < 4 ? PU_DECIDE + lane : PU_CONSTMUT);
-  auto word = [&](uint32_t purpose, int q) { return __shfl_sync(FULL, w.v[q], purpose == PU_CONSTMUT ? 4 : purpose - PU_DECIDE); };
+  auto word = [&](uint32_t purpose, int q) { return g.get(w.v[q], purpose == PU_CONSTMUT ? 4 : purpose - PU_DECIDE); };
   const float u_cross = unit24(word(PU_DECIDE, 0)), u_point = unit24(word(PU_DECIDE, 1));
   const float u_sub = unit24(word(PU_DECIDE, 2)), u_const = unit24(word(PU_DECIDE, 3));
-  __syncwarp();
+  g.sync();
 
   // the child: A[0, sa) ++ B[sb, sb + nb) ++ A[sa + nb - shift, la), all of A without a crossover
   int len = la, sa = la, nb = 0, sb = 0, shift = 0;
@@ -251,7 +280,7 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   if (u_cross < p.cfg.p_cross) {
     const int a = (int)below(word(PU_CROSS, 0), (uint32_t)la);
     const int b = (int)below(word(PU_CROSS, 1), (uint32_t)lb);
-    const int ta = warp_subtree_start(sA, a, lane), tb = warp_subtree_start(sB, b, lane);
+    const int ta = group_subtree_start(g, sA, a), tb = group_subtree_start(g, sB, b);
     const int nl = la - (a - ta + 1) + (b - tb + 1);
     if (nl <= p.Lmax) {
       crossed = true;
@@ -264,7 +293,7 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   }
   uint32_t usedA = 0, usedB = 0;
   const int dB = R + sb - sa;  // B's row follows A's
-  for (int q0 = lane * 4; q0 < len; q0 += 128) {
+  for (int q0 = lane * 4; q0 < len; q0 += 4 * G) {
     uint32_t quad = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -280,11 +309,11 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
     reinterpret_cast<uint32_t *>(out)[q0 >> 2] = quad;
   }
   if (crossed && p.K > 0) {  // slot k takes B's value when only the inserted part reads it
-    usedA = __reduce_or_sync(FULL, usedA);
-    usedB = __reduce_or_sync(FULL, usedB);
+    usedA = __reduce_or_sync(g.mask, usedA);
+    usedB = __reduce_or_sync(g.mask, usedB);
     if (lane < p.K && ((usedB & ~usedA) >> lane & 1u)) c = cb;
   }
-  __syncwarp();
+  g.sync();
 
   if (u_point < p.cfg.p_point) {
     const int t = (int)below(word(PU_POINT, 0), (uint32_t)len);
@@ -299,33 +328,33 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
       const int q = (int)below(w1, (uint32_t)(p.nvars + p.K));
       v = q < p.nvars ? TOK_VAR0 + q : TOK_CONST0 + (q - p.nvars);
     }
-    __syncwarp();
+    g.sync();
     if (lane == 0) out[t] = (uint8_t)v;
-    __syncwarp();
+    g.sync();
   }
 
   if (u_sub < p.cfg.p_subtree && p.cfg.max_subtree > 0) {
     const int t = (int)below(word(PU_SUBTREE, 0), (uint32_t)len);
     const int n = 1 + (int)below(word(PU_SUBTREE, 1), (uint32_t)p.cfg.max_subtree);
-    const int s = warp_subtree_start(out, t, lane);
+    const int s = group_subtree_start(g, out, t);
     const int span = t - s + 1, nl = len - span + n;
     if (nl <= p.Lmax) {
       // out[0, s) ++ n new tokens ++ out[t + 1, len), built where A's row was
-      for (int q = lane; q < nl; q += 32)
+      for (int q = lane; q < nl; q += G)
         if (q < s || q >= s + n) sA[q] = out[q < s ? q : q + span - n];
       int d = 0;
-      for (int q0 = 0; q0 < n; q0 += 32) {
-        const Word4 g = rng.draw((uint32_t)(q0 + lane), (uint32_t)i, PU_SUBGEN);
-        for (int q = q0; q < n && q < q0 + 32; ++q) {
-          const int v = gen_token(d, n - q, p.nvars, p.K, p.cfg.unary_ops, __shfl_sync(FULL, g.v[0], q - q0),
-                                  __shfl_sync(FULL, g.v[1], q - q0));
+      for (int q0 = 0; q0 < n; q0 += G) {
+        const Word4 d4 = rng.draw((uint32_t)(q0 + lane), (uint32_t)i, PU_SUBGEN);
+        for (int q = q0; q < n && q < q0 + G; ++q) {
+          const int v = gen_token(d, n - q, p.nvars, p.K, p.cfg.unary_ops, g.get(d4.v[0], q - q0),
+                                  g.get(d4.v[1], q - q0));
           if (lane == 0) sA[s + q] = (uint8_t)v;
           d += effect(v);
         }
       }
       len = nl;
       out = sA;
-      __syncwarp();
+      g.sync();
     }
   }
 
@@ -339,7 +368,7 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
   uint8_t *g_out = p.prog_out + (size_t)i * p.Lmax;
   const int ograin = row_grain(p.prog_out, p.Lmax);
   if (ograin == 1) {
-    for (int t = lane; t < p.Lmax; t += 32) g_out[t] = t < len ? out[t] : 0;
+    for (int t = lane; t < p.Lmax; t += G) g_out[t] = t < len ? out[t] : 0;
   } else {
     auto quad = [&](int t4) {  // bytes 4 t4 .. 4 t4 + 3
       const int left = len - 4 * t4;
@@ -347,11 +376,10 @@ __global__ void __launch_bounds__(VARY_WARPS * 32) vary_kernel(VaryParams p) {
       return left >= 4 ? v : (left <= 0 ? 0u : v & ((1u << (8 * left)) - 1u));
     };
     if (ograin == 16) {
-      if (lane * 16 < p.Lmax)
-        reinterpret_cast<uint4 *>(g_out)[lane] =
-            make_uint4(quad(4 * lane), quad(4 * lane + 1), quad(4 * lane + 2), quad(4 * lane + 3));
+      for (int t = lane; t * 16 < p.Lmax; t += G)
+        reinterpret_cast<uint4 *>(g_out)[t] = make_uint4(quad(4 * t), quad(4 * t + 1), quad(4 * t + 2), quad(4 * t + 3));
     } else {
-      for (int t = lane; 4 * t < p.Lmax; t += 32) reinterpret_cast<uint32_t *>(g_out)[t] = quad(t);
+      for (int t = lane; 4 * t < p.Lmax; t += G) reinterpret_cast<uint32_t *>(g_out)[t] = quad(t);
     }
   }
   if (lane == 0) p.len_out[i] = len;
@@ -508,8 +536,9 @@ sr_status sr_vary(sr_ctx *ctx, const uint8_t *prog_in, const int32_t *len_in, co
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
   VaryParams vp{prog_in, len_in, c_in, parents, prog_out, len_out, c_out, P, Lmax, K, nvars, *cfg,
                 make_rng(seed, gen, ctx->gen_dev), P_in};
-  SR_CHECK_CUDA(ctx, launch(vary_kernel, (P + VARY_WARPS - 1) / VARY_WARPS, VARY_WARPS * 32,
-                            VARY_WARPS * 3 * vary_row_bytes(Lmax), ctx->stream, vp));
+  const int lanes = vary_halves(P, Lmax) ? 16 : 32, per = VARY_THREADS / lanes;
+  SR_CHECK_CUDA(ctx, launch(lanes == 16 ? vary_kernel<16> : vary_kernel<32>, (P + per - 1) / per, VARY_THREADS,
+                            per * 3 * vary_row_bytes(Lmax), ctx->stream, vp));
   SR_CHECK_CUDA(ctx, cudaGetLastError());
   ctx->launches += 1;
   return SR_OK;
