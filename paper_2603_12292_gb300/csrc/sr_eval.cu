@@ -438,35 +438,39 @@ __device__ __forceinline__ int p2p_case(float yh, float y, int M, float Mf, floa
 // Eq. 2 sums over one lane's 8 cases (nvalid of them inside the chunk):
 // pairs with both values finite give the moments of the shifted output d
 // and the centred target e; one invalid value counts in n1, both in n2.
-// Out of line: the copy inside the interpreter loop measured 1.7 % slower.
+// Four values at a time, so that these sums and the interpreter's operators stay
+// in the instruction cache together (the only copy is inside `accumulate`): 4,096 x
+// 100,000 with the base operators 6,120 -> 5,605 us, a population under way 5,357 ->
+// 4,970, all operators 2,048 x 50,001 2,115 -> 2,064 (the eight at once and inline:
+// 5,940, 5,207, 2,066).
 struct R4Part { float s1, s2, s3, s4, s5; int n1, n2; };
-__device__ __noinline__ R4Part r4_part(V8 T, float4 ya, float4 yb, int nvalid, float shift) {
+__device__ __forceinline__ R4Part r4_part(V8 T, float4 ya, float4 yb, int nvalid, float shift) {
   float tv[CPL];
   unpack8(T, tv);
-  const float yv[CPL] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-  float d[CPL], e[CPL];
-  int c1 = 0, c2 = 0;
+  float t0 = tv[0], t1 = tv[1], t2 = tv[2], t3 = tv[3], y0 = ya.x, y1 = ya.y, y2 = ya.z, y3 = ya.w;
+  R4Part r{0.f, 0.f, 0.f, 0.f, 0.f, 0, 0};
+#pragma unroll 1
+  for (int h = 0; h < CPL; h += 4) {
+    const float t[4] = {t0, t1, t2, t3}, y[4] = {y0, y1, y2, y3};
+    float d[4], e[4];
 #pragma unroll
-  for (int i = 0; i < CPL; ++i) {
-    const bool ok = i < nvalid;
-    const bool vh = isfinite(tv[i]), vy = isfinite(yv[i]);
-    const bool pair = ok && vh && vy;
-    c1 += (ok && vh != vy) ? 1 : 0;
-    c2 += (ok && !vh && !vy) ? 1 : 0;
-    d[i] = pair ? tv[i] - shift : 0.0f;
-    e[i] = pair ? yv[i] : 0.0f;
+    for (int i = 0; i < 4; ++i) {
+      const bool ok = h + i < nvalid;
+      const bool vh = isfinite(t[i]), vy = isfinite(y[i]);
+      const bool pair = ok && vh && vy;
+      r.n1 += (ok && vh != vy) ? 1 : 0;
+      r.n2 += (ok && !vh && !vy) ? 1 : 0;
+      d[i] = pair ? t[i] - shift : 0.0f;
+      e[i] = pair ? y[i] : 0.0f;
+    }
+    r.s1 += (d[0] + d[1]) + (d[2] + d[3]);
+    r.s2 += (d[0] * d[0] + d[1] * d[1]) + (d[2] * d[2] + d[3] * d[3]);
+    r.s3 += (d[0] * e[0] + d[1] * e[1]) + (d[2] * e[2] + d[3] * e[3]);
+    r.s4 += (e[0] + e[1]) + (e[2] + e[3]);
+    r.s5 += (e[0] * e[0] + e[1] * e[1]) + (e[2] * e[2] + e[3] * e[3]);
+    t0 = tv[4]; t1 = tv[5]; t2 = tv[6]; t3 = tv[7];
+    y0 = yb.x; y1 = yb.y; y2 = yb.z; y3 = yb.w;
   }
-  R4Part r;
-  r.s1 = ((d[0] + d[1]) + (d[2] + d[3])) + ((d[4] + d[5]) + (d[6] + d[7]));
-  r.s2 = ((d[0] * d[0] + d[1] * d[1]) + (d[2] * d[2] + d[3] * d[3])) +
-         ((d[4] * d[4] + d[5] * d[5]) + (d[6] * d[6] + d[7] * d[7]));
-  r.s3 = ((d[0] * e[0] + d[1] * e[1]) + (d[2] * e[2] + d[3] * e[3])) +
-         ((d[4] * e[4] + d[5] * e[5]) + (d[6] * e[6] + d[7] * e[7]));
-  r.s4 = ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-  r.s5 = ((e[0] * e[0] + e[1] * e[1]) + (e[2] * e[2] + e[3] * e[3])) +
-         ((e[4] * e[4] + e[5] * e[5]) + (e[6] * e[6] + e[7] * e[7]));
-  r.n1 = c1;
-  r.n2 = c2;
   return r;
 }
 
