@@ -40,7 +40,7 @@ KERNEL_SOURCES = {
     "eval": ("sr_eval.cu", "sr_vm.cuh", "sr_decode.cuh", "sr_interp.cuh", "sr_common.cuh"),
     "grad": ("sr_grad.cu", "sr_gradvm.cuh", "sr_vm.cuh", "sr_decode.cuh", "sr_interp.cuh", "sr_common.cuh"),
 }
-# Dominant kernels of the workloads, each from one ncu --set full capture
+# Dominant kernels of the workloads, each from one ncu capture
 # summarised under profiles/: the captured workload, DRAM bytes (read +
 # write) of the captured launch, the units (node-evaluations) it processed,
 # smsp__issue_active, the summary file, and the hash of the kernel's sources
@@ -48,25 +48,25 @@ KERNEL_SOURCES = {
 # workload, and for another size only where it grows with the units (scale).
 KERNEL_NCU = {
     # eval_kernel<MODE_BOTH> on the headline workload, inputs read once
-    "paper": {"workload": "paper-4096x100k", "dram_bytes": 173.062e6 + 11.567e6, "units": None,
-              "issue_active": 0.839, "scale": False, "sources": "eval",
-              "capture": "profiles/eval_kernel_paper-4096x100k.md", "src": "a0bec70a9304581f"},
-    # grad_kernel: the tape write-back evicted from L2 grows with the units
-    "grad": {"workload": "adjoint-2048x131072", "dram_bytes": 4.489e9 + 18.163e9, "units": 1.3324e10,
-             "issue_active": 0.726, "scale": True, "sources": "grad",
-             "capture": "profiles/grad_kernel_adjoint-2048x131072.md", "src": "9914c98e792aff67"},
+    "paper": {"workload": "paper-4096x100k", "dram_bytes": 174.839e6 + 18.818e6, "units": None,
+              "issue_active": 0.822, "scale": False, "sources": "eval",
+              "capture": "profiles/eval_kernel_paper-4096x100k.md", "src": "d5ac140bcea09971"},
+    # grad_kernel: the write-back of the tape's lines grows with the units
+    "grad": {"workload": "adjoint-2048x131072", "dram_bytes": 0.019e9 + 1.687e9, "units": 1.3324e10,
+             "issue_active": 0.630, "scale": True, "sources": "grad",
+             "capture": "profiles/grad_kernel_adjoint-2048x131072.md", "src": "89927252563fb735"},
     # eval_kernel<R4>: inputs read once (L2-resident), at the full size
-    "beagle": {"workload": "beagle-4096x100k", "dram_bytes": 171.088e6 + 11.973e6, "units": 2.3977e10,
-               "issue_active": 0.817, "scale": False, "sources": "eval",
-               "capture": "profiles/eval_kernel_r4_beagle-4096x100k.md", "src": "a0bec70a9304581f"},
+    "beagle": {"workload": "beagle-4096x100k", "dram_bytes": 171.639e6 + 15.667e6, "units": 2.3977e10,
+               "issue_active": 0.822, "scale": False, "sources": "eval",
+               "capture": "profiles/eval_kernel_r4_beagle-4096x100k.md", "src": "d5ac140bcea09971"},
     # eval_batched_kernel: the first 8 problems; inputs read once
-    "batched": {"workload": "batched-8", "dram_bytes": 1625.761e6 + 47.885e6, "units": 4.0723e11,
-                "issue_active": 0.816, "scale": False, "sources": "eval",
-                "capture": "profiles/eval_batched_kernel_batched-8.md", "src": "a0bec70a9304581f"},
+    "batched": {"workload": "batched-8", "dram_bytes": 2036.080e6 + 174.584e6, "units": 4.0723e11,
+                "issue_active": 0.806, "scale": False, "sources": "eval",
+                "capture": "profiles/eval_batched_kernel_batched-8.md", "src": "d5ac140bcea09971"},
     # eval_kernel<CORR> at Lmax 256: inputs read once
-    "large": {"workload": "large-16384x131072", "dram_bytes": 402.477e6 + 20.297e6, "units": 2.5087e11,
-              "issue_active": 0.820, "scale": False, "sources": "eval",
-              "capture": "profiles/eval_kernel_corr_large-16384x131072.md", "src": "a0bec70a9304581f"},
+    "large": {"workload": "large-16384x131072", "dram_bytes": 511.023e6 + 80.748e6, "units": 2.5087e11,
+              "issue_active": 0.793, "scale": False, "sources": "eval",
+              "capture": "profiles/eval_kernel_corr_large-16384x131072.md", "src": "d5ac140bcea09971"},
 }
 
 
