@@ -166,9 +166,7 @@ inline int chunk_minb(int Lmax, int tuned) {  // eval_minb by the same rule
 }
 
 // ---------------------------------------------------------------- operators
-__device__ __forceinline__ float4 ldx4(const float *p) {
-  return __ldg(reinterpret_cast<const float4 *>(p));
-}
+__device__ __forceinline__ float4 ldx4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -197,12 +195,12 @@ __device__ double block_sum(double v, double *red) {
 
 // FP64 sum and count of one chunk of y: every value, or (finite_only) the
 // finite ones.  ysum [nchunks][2].
-__device__ void ysum_chunk(const float *__restrict__ y, int N, int chunk, int c, bool finite_only,
+__device__ void ysum_chunk(const float *y, int N, int chunk, int c, bool finite_only,
                            double *ysum, double *red) {
   const int beg = c * chunk, end = min(N, beg + chunk);
   double a = 0.0, n = 0.0;
   for (int i = beg + threadIdx.x; i < end; i += blockDim.x) {
-    const float v = __ldg(y + i);
+    const float v = y[i];
     if (!finite_only || isfinite(v)) {
       a += (double)v;
       n += 1.0;
@@ -219,7 +217,7 @@ __device__ void ysum_chunk(const float *__restrict__ y, int N, int chunk, int c,
 // ybar = (sum of the chunk sums) / (their count), chunks in order; then
 // yc = fl32(y - ybar) on one chunk (NaN at invalid targets when
 // nan_invalid) with the chunk's FP64 sum and sum of squares of yc
-__device__ void ycenter_chunk(const float *__restrict__ y, int N, int chunk, int nchunks, int c,
+__device__ void ycenter_chunk(const float *y, int N, int chunk, int nchunks, int c,
                               const double *ysum, bool nan_invalid, float *yc, double *ychunk,
                               double *red) {
   __shared__ double ybar_s;
@@ -346,8 +344,8 @@ static __device__ __noinline__ float4 unary4(int tok, float4 x) {
   }
 #undef SR_EACH
 }
-__device__ void xform_block(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt, int depth,
-                            const uint8_t *__restrict__ xneed, float *__restrict__ xt, int block, int j, int part) {
+__device__ void xform_block(const float *X, long long ldx, int nvars, int N, int ldxt, int depth,
+                            const uint8_t *xneed, float *xt, int block, int j, int part) {
   const int c = (block * XF_THREADS + threadIdx.x) * 4;
   if (c >= N) return;  // c + 3 < ldx and < ldxt: both are multiples of 4 and >= N
   const float4 x = ldx4(X + (size_t)j * ldx + c);
@@ -384,8 +382,8 @@ __global__ void __launch_bounds__(PREP_THREADS) ycenter_kernel(CenterParams y) {
 }
 // The first yblocks blocks centre the target, one chunk each.
 __global__ void __launch_bounds__(XF_THREADS)
-    xform_kernel(const float *__restrict__ X, long long ldx, int nvars, int N, int ldxt, int depth,
-                 const uint8_t *__restrict__ xneed, float *__restrict__ xt, int yblocks, CenterParams y) {
+    xform_kernel(const float *X, long long ldx, int nvars, int N, int ldxt, int depth, const uint8_t *xneed, float *xt,
+                 int yblocks, CenterParams y) {
   __shared__ double red[XF_THREADS / 32];
   launch_wait();
   const int block = (int)blockIdx.x - yblocks, per_part = (N + XF_THREADS * 4 - 1) / (XF_THREADS * 4);
@@ -413,8 +411,8 @@ struct Kahan {
 
 __device__ __forceinline__ float sel(bool ok, float v) { return ok ? v : 0.0f; }
 
-__device__ __forceinline__ float4 load_y4(const float *__restrict__ y, int c0, int N) {
-  if (c0 + 3 < N) return __ldg(reinterpret_cast<const float4 *>(y + c0));
+__device__ __forceinline__ float4 load_y4(const float *y, int c0, int N) {
+  if (c0 + 3 < N) return ldx4(y + c0);
   float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c0 < N) r.x = y[c0];
   if (c0 + 1 < N) r.y = y[c0 + 1];
@@ -503,7 +501,7 @@ struct Acc {
 // N values; yc: the centred target (1 - r^2, Eq. 2).
 template <int MODE>
 __device__ __noinline__ void accumulate(Acc *acc, V8 T, int c0, int cl, int cl4, int cend, int first,
-                                  const float *__restrict__ y, const float *__restrict__ yc, int N, int want, int M) {
+                                  const float *y, const float *yc, int N, int want, int M) {
   const bool do_mse = MODE == MODE_MSE || (MODE == MODE_BOTH && (want & 1));
   const bool do_corr = MODE == MODE_CORR || (MODE == MODE_BOTH && (want & 2));
   float tv[CPL];

@@ -120,8 +120,7 @@ __device__ __forceinline__ unsigned long long order_key(double f) {
 // tournaments of 4 over 262,144 fitnesses: 17.2 us with FP64 compares and one
 // read after the other, now 11.4 (the gather's latency).
 template <int MAXIMISE>
-__global__ void tournament_kernel(const double *__restrict__ fitness, int P, int k, Rng rng_in,
-                                  int32_t *__restrict__ parents) {
+__global__ void tournament_kernel(const double *fitness, int P, int k, Rng rng_in, int32_t *parents) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * P) return;
   launch_wait();
@@ -136,7 +135,7 @@ __global__ void tournament_kernel(const double *__restrict__ fitness, int P, int
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       cand[q] = (int)below(w.v[q], (uint32_t)P);
-      f[q] = __ldg(fitness + cand[q]);  // (in range for the words past k too)
+      f[q] = fitness[cand[q]];  // (in range for the words past k too)
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -193,12 +192,12 @@ template <int G>
 __device__ __forceinline__ void load_row(uint8_t *dst, const uint8_t *src, int n, int grain, int lane) {
   if (grain == 16) {
     for (int t = lane; t * 16 < n; t += G)
-      reinterpret_cast<uint4 *>(dst)[t] = __ldg(reinterpret_cast<const uint4 *>(src) + t);
+      reinterpret_cast<uint4 *>(dst)[t] = reinterpret_cast<const uint4 *>(src)[t];
   } else if (grain == 4) {
     for (int t = lane; t * 4 < n; t += G)
-      reinterpret_cast<uint32_t *>(dst)[t] = __ldg(reinterpret_cast<const uint32_t *>(src) + t);
+      reinterpret_cast<uint32_t *>(dst)[t] = reinterpret_cast<const uint32_t *>(src)[t];
   } else {
-    for (int t = lane; t < n; t += G) dst[t] = __ldg(src + t);
+    for (int t = lane; t < n; t += G) dst[t] = src[t];
   }
 }
 

@@ -154,7 +154,7 @@ __device__ __forceinline__ void grad_item(const GradParams &p, int c, int prog, 
 #pragma unroll
     for (int i = 0; i < GCPL; ++i) {
       const bool ok = (okm >> i) & 1u;
-      e[i] = ok ? t[i] - __ldg(p.y + c0 + i) : 0.0f;
+      e[i] = ok ? t[i] - p.y[c0 + i] : 0.0f;
       e2 += e[i] * e[i];
     }
     se.add(e2);
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(GFINAL_THREADS) grad_finalize_kernel(GradFinal
 // work spreads over the SMs (8 steps on 24 tables of 2,048 constants with their
 // gradients: 745 us with 256 threads a block, 733 with 64).
 constexpr int ADAM_THREADS = 64;
-__device__ __forceinline__ void adam_one(float *c, const double *__restrict__ g, double *m, double *v, int i,
+__device__ __forceinline__ void adam_one(float *c, const double *g, double *m, double *v, int i,
                                          double lr, double b1, double b2, double eps, double bc1, double bc2) {
   const double gi = g[i];
   if (!isfinite(gi)) return;  // leaves c, m, v unchanged
@@ -313,7 +313,7 @@ __device__ __forceinline__ void adam_one(float *c, const double *__restrict__ g,
   c[i] = __double2float_rn(__dsub_rn((double)c[i], step));
 }
 
-__global__ void adam_kernel(float *c, const double *__restrict__ g, double *m, double *v, int n,
+__global__ void adam_kernel(float *c, const double *g, double *m, double *v, int n,
                             double lr, double b1, double b2, double eps, double bc1, double bc2) {
   launch_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

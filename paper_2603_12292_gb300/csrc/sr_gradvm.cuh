@@ -491,7 +491,7 @@ __device__ __forceinline__ V4 pack4(const float (&t)[GCPL]) { return V4{{pack(t[
 // the forward loop), %6 tape, then %7 slot 0 and %8 row 0 of this lane; the
 // reverse loop has %7-%8 its X register (RV_DIVT2) and %9, %10 those.
 // clang-format off
-#define GR_ROW(d0, d1, xa) "mad.wide.u32 a, wy, 4, " xa ";\n\tld.global.nc.v2.b64 {" d0 ", " d1 "}, [a];\n\t"
+#define GR_ROW(d0, d1, xa) "mad.wide.u32 a, wy, 4, " xa ";\n\tld.global.v2.b64 {" d0 ", " d1 "}, [a];\n\t"
 #define GR_SLOT(st) "bfe.u32 s, wx, 8, 16;\n\tadd.u32 s, s, " st ";\n\t"
 #define GR_SPLAT(d0, d1) "mov.b64 " d0 ", {wy, wy};\n\tmov.b64 " d1 ", " d0 ";\n\t"
 #define GR_PUSH(s0, s1) "st.global.v2.b64 [%6], {" s0 ", " s1 "};\n\tadd.u64 %6, %6, 512;\n\t"

@@ -201,15 +201,15 @@ __device__ __noinline__ V8 ext8(uint32_t op, V8 v) {
   "ld.shared.v2.b32 {wx, wy}, [%8];\n\tadd.u32 %8, %8, 8;\n\tand.b32 %9, wx, 255;\n\t" \
   "brx.idx.uni %9, TABLE;\n\t"
 #define SR_LDX_WIDE \
-  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.nc.v4.b64 {%4, %5, %6, %7}, [a];\n\t"
+  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.v4.b64 {%4, %5, %6, %7}, [a];\n\t"
 #define SR_LDT_WIDE \
-  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.nc.v4.b64 {%0, %1, %2, %3}, [a];\n\t"
+  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.v4.b64 {%0, %1, %2, %3}, [a];\n\t"
 #define SR_LDX_HALVES \
-  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.nc.v2.b64 {%4, %5}, [a];\n\t" \
-  "mad.wide.u32 a, wy, 4, %12;\n\tld.global.nc.v2.b64 {%6, %7}, [a];\n\t"
+  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.v2.b64 {%4, %5}, [a];\n\t" \
+  "mad.wide.u32 a, wy, 4, %12;\n\tld.global.v2.b64 {%6, %7}, [a];\n\t"
 #define SR_LDT_HALVES \
-  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.nc.v2.b64 {%0, %1}, [a];\n\t" \
-  "mad.wide.u32 a, wy, 4, %12;\n\tld.global.nc.v2.b64 {%2, %3}, [a];\n\t"
+  "mad.wide.u32 a, wy, 4, %11;\n\tld.global.v2.b64 {%0, %1}, [a];\n\t" \
+  "mad.wide.u32 a, wy, 4, %12;\n\tld.global.v2.b64 {%2, %3}, [a];\n\t"
 #define SR_SLOT "shr.u32 s, wx, 8;\n\tadd.u32 s, s, %10;\n\t"
 #define SR_LDS SR_SLOT "ld.shared.v2.b64 {%4, %5}, [s];\n\tld.shared.v2.b64 {%6, %7}, [s + 512];\n\t"
 #define SR_STS SR_SLOT "st.shared.v2.b64 [s], {%0, %1};\n\tst.shared.v2.b64 [s + 512], {%2, %3};\n\t"
@@ -298,8 +298,8 @@ struct Shape {
 // 256-bit load a row); else two 128-bit loads.
 // LEAN: the code around it is large, or runs nearly as often (Shape).
 template <bool EXT, bool WIDE, bool LEAN>
-__device__ __forceinline__ V8 interpret(const uint2 *code, const char *stk, const float *__restrict__ xa,
-                                        const float *__restrict__ xb) {
+__device__ __forceinline__ V8 interpret(const uint2 *code, const char *stk, const float *xa,
+                                        const float *xb) {
   using S = Shape<EXT, LEAN>;
   V8 T = splat8(0.f), X;
   uint32_t ip = (uint32_t)__cvta_generic_to_shared(code), op;
