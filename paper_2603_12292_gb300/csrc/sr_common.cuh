@@ -124,10 +124,6 @@ bool stream_capturing(sr_ctx *ctx);
 // device) pair once per process (thread-safe).
 sr_status allow_dynamic_smem(sr_ctx *ctx, const void *kernel);
 
-// A number no other call of the process has (not 0): a call's kernels note something for
-// each other by storing it, so that nothing has to be cleared first.
-unsigned long long call_tag();
-
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // sequential carving of the workspace

@@ -3,7 +3,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <atomic>
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -24,11 +23,6 @@ sr_status fail(sr_ctx *ctx, sr_status s, const char *fmt, ...) {
 
 sr_status cuda_fail(sr_ctx *ctx, cudaError_t e, const char *what) {
   return fail(ctx, SR_ECUDA, "%s: %s", what, cudaGetErrorString(e));
-}
-
-unsigned long long call_tag() {
-  static std::atomic<unsigned long long> calls{0};
-  return ++calls;
 }
 
 bool stream_capturing(sr_ctx *ctx) {
@@ -71,6 +65,8 @@ sr_status ensure_workspace(sr_ctx *ctx, size_t bytes) {
                 cudaGetErrorString(e));
   }
   ctx->ws_bytes = want;
+  // the notes that a call's kernels leave for each other start clear
+  SR_CHECK_CUDA(ctx, cudaMemsetAsync(ctx->ws, 0, 256, ctx->stream));
   return SR_OK;
 }
 

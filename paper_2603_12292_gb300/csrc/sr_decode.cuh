@@ -269,8 +269,8 @@ __device__ inline void decode_eval_warp(const DecodeArgs &p, int prog, unsigned 
     p.flags[prog] = deep ? SR_PF_TOO_DEEP : 0;
     const bool past_cap = used > p.cap_slots;
     p.ncode[prog] = deep ? 0 : s.cnt[L - 1] | (ext ? NCODE_EXT : 0) | (past_cap ? NCODE_DEEP : 0);
-    if (!deep && ext) *p.ext_note = p.tag;
-    if (!deep && past_cap) *p.deep_note = p.tag;
+    if (!deep && ext) *p.ext_note = 1;
+    if (!deep && past_cap) *p.deep_note = 1;
   }
 }
 

@@ -94,11 +94,10 @@ struct EvalParams {
   int32_t *flags;          // [P]
   uint2 *code;             // [P][Lmax] decoded instructions
   int32_t *ncode;          // [P]
-  // [0] work counter, [1] work counter of the EXT pass, [2] `tag` when it has
-  // programs, [3], [4] the same of the deep pass; the decode launch zeroes the
-  // counters and notes the tags
+  // [0] work counter, [1] work counter of the EXT pass, [2] the decoder's note that
+  // it has programs, [3], [4] the same of the deep pass, [5], [6] the notes as the
+  // later passes read them (hand_over)
   unsigned long long *queue;
-  unsigned long long tag;  // call_tag
   float *yhat;             // predict: [P][ldy]
   long long ldy;
   int warp_bytes;          // shared memory per warp
@@ -276,7 +275,6 @@ __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_s
   a.cap_slots = cap_slots;
   a.ext_note = p.queue + 2;
   a.deep_note = p.queue + 4;
-  a.tag = p.tag;
   a.xform = p.xform;
   a.xneed = p.xneed;
   return a;
@@ -684,10 +682,20 @@ __device__ __forceinline__ bool takes(int pass, int ncode) {
   if (ncode_deep(ncode)) return false;
   return pass == PASS_SHALLOW || ncode_ext(ncode) == (pass == PASS_EXT);
 }
+// The first pass (base or shallow) hands the decoder's notes over to the passes
+// after it and clears them for the next call.  A replay of a captured call then
+// makes a pass only when its own programs need it (a note that stayed had every
+// replay after it walk the items of an empty pass).
+__device__ __forceinline__ void hand_over(unsigned long long *queue) {
+  queue[5] = queue[2];
+  queue[6] = queue[4];
+  queue[2] = queue[4] = 0;
+}
 // the pass's work counter; NULL when it has no programs
-__device__ __forceinline__ unsigned long long *pass_queue(unsigned long long *queue, int pass, unsigned long long tag) {
-  if (pass == PASS_EXT) return queue[2] == tag ? queue + 1 : nullptr;
-  if (pass == PASS_DEEP) return queue[4] == tag ? queue + 3 : nullptr;
+__device__ __forceinline__ unsigned long long *pass_queue(unsigned long long *queue, int pass) {
+  if (pass == PASS_EXT) return queue[5] ? queue + 1 : nullptr;
+  if (pass == PASS_DEEP) return queue[6] ? queue + 3 : nullptr;
+  if (blockIdx.x == 0 && threadIdx.x == 0) hand_over(queue);
   return queue;
 }
 
@@ -696,7 +704,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_kernel(EvalParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   launch_wait();
   const int pass = EXT ? p.pass : PASS_BASE;
-  unsigned long long *q = pass_queue(p.queue, pass, p.tag);
+  unsigned long long *q = pass_queue(p.queue, pass);
   if (!q) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, p.warp_bytes, p.slots);
@@ -748,7 +756,6 @@ struct BatchParams {
   int total_progs;
   long long total_items;
   unsigned long long *queue;  // as EvalParams::queue
-  unsigned long long tag;
   int warp_bytes;
   int slots;
   int maxL;                   // the largest Lmax of the batch
@@ -827,7 +834,6 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const
   }
   EvalParams p = view(b.prob[lo]);
   p.queue = b.queue;
-  p.tag = b.tag;
   decode_eval_warp(decode_args(p, b.slots), g - b.prob[lo].prog_begin,
                    dsm + (size_t)warp * decode_scratch_bytes(b.maxL));
 }
@@ -848,7 +854,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) eval_batched_kernel(const __
   extern __shared__ __align__(16) unsigned char smem[];
   launch_wait();
   const int pass = EXT ? b.pass : PASS_BASE;
-  unsigned long long *qc = pass_queue(b.queue, pass, b.tag);
+  unsigned long long *qc = pass_queue(b.queue, pass);
   if (!qc) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const WarpSmem w = warp_smem(smem, warp, b.warp_bytes, b.slots);
@@ -1277,7 +1283,6 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   ep.code = reinterpret_cast<uint2 *>(ws + pl.off_code);
   ep.ncode = reinterpret_cast<int32_t *>(ws + pl.off_ncode);
   ep.queue = reinterpret_cast<unsigned long long *>(ws + pl.off_queue);
-  ep.tag = call_tag();
   ep.yhat = yhat;
   ep.ldy = ldy;
   ep.slots = pl.slots;
@@ -1553,7 +1558,6 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
     const size_t g1 = std::min(order.size(), g0 + MAX_BATCH);
     BatchParams b;
     group_bytes(g0, g1, &b);
-    b.tag = call_tag();
     for (int r = 0; r < b.nprob; ++r)
       if (b.prob[r].xform)
         SR_CHECK_CUDA(ctx, cudaMemsetAsync(b.prob[r].xneed, 0,

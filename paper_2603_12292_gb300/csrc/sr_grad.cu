@@ -52,11 +52,11 @@ struct GradParams {
   int32_t *flags;     // [P]
   uint2 *code;        // [P][grad_code_words(Lmax)] forward, then reverse program
   int32_t *nfwd, *nrev;  // [P] their words
-  // [0] work counter, [1] work counter of the big pass, [2] `tag` when some
-  // program's code is longer than the first pass's share (the big pass takes
-  // those, with room for any); the decode launch zeroes the counters
+  // [0] work counter, [1] work counter of the big pass, [2] the decoder's note that
+  // some program's code is longer than the first pass's share (the big pass takes
+  // those, with room for any), [5] the note as that pass reads it (grad_pass);
+  // the decode launch zeroes the counters
   unsigned long long *queue;
-  unsigned long long tag;  // call_tag
   int cap;            // code words per warp of this launch
   int big;            // 1: the big pass
   char *gtape;        // per warp: Lmax entries of GSLOT bytes
@@ -73,9 +73,9 @@ __host__ __device__ inline int grad_warp_bytes(int Lmax, int K, int words) {
 // evolved populations have at most about 1.9 words a token
 __host__ __device__ inline int grad_cap_words(int Lmax) { return 2 * Lmax + 8; }
 
-__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *queue, unsigned long long tag) {
+__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *queue) {
   return GradDecode{p.programs, p.lengths, p.consts, p.Lmax, p.K, p.nvars, p.ldx, p.code, p.nfwd, p.nrev, p.flags,
-                    grad_cap_words(p.Lmax), queue + 2, tag};
+                    grad_cap_words(p.Lmax), queue + 2};
 }
 
 // a warp per program
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_kernel(GradPara
   if (blockIdx.x == 0 && threadIdx.x < 2) p.queue[threadIdx.x] = 0;
   const int warp = threadIdx.x >> 5, prog = blockIdx.x * DECODE_WARPS + warp;
   if (prog < p.P)
-    decode_grad_warp(grad_decode_args(p, p.queue, p.tag), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
+    decode_grad_warp(grad_decode_args(p, p.queue), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
                      slots_for(p.Lmax));
 }
 
@@ -175,12 +175,24 @@ __device__ __forceinline__ bool grad_takes(const GradParams &p, int prog, int bi
   return nf > 0 && ((nf + p.nrev[prog] > grad_cap_words(p.Lmax)) == (big != 0));
 }
 
+// Whether a pass has programs.  The first hands the decoder's note over to the big
+// pass and clears it for the next call, so that a replay of a captured call walks
+// the big pass's items only when its own programs need it.
+__device__ __forceinline__ bool grad_pass(unsigned long long *queue, int big) {
+  if (big) return queue[5] != 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    queue[5] = queue[2];
+    queue[2] = 0;
+  }
+  return true;
+}
+
 // Two passes over the work items: the second (big) for the programs whose code
 // does not fit the first's share, which returns at once when there are none.
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_kernel(GradParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
   launch_wait();
-  if (p.big && p.queue[2] != p.tag) return;
+  if (!grad_pass(p.queue, p.big)) return;
   const int lane = threadIdx.x & 31;
   const GradWarp w = grad_warp(smem, p.Lmax, p.K, p.cap, p.gtape);
   for (;;) {
@@ -203,7 +215,7 @@ struct GradBatch {
   double *dconst[MAX_GBATCH];
   int nprob, total_progs;
   long long total_items;
-  unsigned long long *queue, tag;
+  unsigned long long *queue;
   char *gtape;
   const int32_t *abort;
   unsigned *err;
@@ -231,7 +243,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(
   if (g >= b.total_progs) return;
   int q = 0;
   while (q + 1 < b.nprob && b.prog_begin[q + 1] <= g) ++q;
-  decode_grad_warp(grad_decode_args(b.prob[q], b.queue, b.tag), g - b.prog_begin[q],
+  decode_grad_warp(grad_decode_args(b.prob[q], b.queue), g - b.prog_begin[q],
                    dsm + (size_t)warp * grad_scratch_bytes(b.Lw), slots_for(b.prob[q].Lmax));
 }
 
@@ -241,7 +253,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_batched_kernel(const __grid_constant__ GradBatch b) {
   extern __shared__ __align__(16) unsigned char smem[];
   launch_wait();
-  if (b.big && b.queue[2] != b.tag) return;
+  if (!grad_pass(b.queue, b.big)) return;
   const int lane = threadIdx.x & 31;
   const GradWarp w = grad_warp(smem, b.Lw, b.Kw, b.cap, b.gtape);
   for (;;) {
@@ -459,7 +471,6 @@ sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *leng
   gp.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
   gp.nrev = gp.nfwd + P;
   gp.queue = reinterpret_cast<unsigned long long *>(ws + off_q);
-  gp.tag = call_tag();
   gp.gtape = ws + off_t;
   gp.abort = ctx->abort_flag;
   gp.err = ctx->dev_words;
@@ -557,7 +568,6 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
         p.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
         p.nrev = p.nfwd + q.P;
         p.queue = nullptr;
-        p.tag = 0;
         p.gtape = nullptr;
         p.abort = nullptr;
         p.err = nullptr;
@@ -576,7 +586,6 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
       b->total_progs = progs;
       b->total_items = items;
       b->queue = reinterpret_cast<unsigned long long *>(ctx->ws + off_q);
-      b->tag = call_tag();
       b->gtape = ctx->ws + off_t;
       b->abort = ctx->abort_flag;
       b->err = ctx->dev_words;

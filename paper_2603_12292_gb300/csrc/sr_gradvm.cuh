@@ -156,8 +156,8 @@ struct GradDecode {
   uint2 *code;              // [P][grad_code_words(Lmax)]: forward, then reverse
   int32_t *nfwd, *nrev;     // [P] words of each (with its end marker); nfwd 0: invalid
   int32_t *flags;           // [P]
-  int cap_words;            // *big_note is set to `tag` when some program has more words than this
-  unsigned long long *big_note, tag;
+  int cap_words;            // *big_note is set to 1 when some program has more words than this
+  unsigned long long *big_note;
 };
 
 // info[] of a token, beside the need: what its subtree reads
@@ -472,7 +472,7 @@ __device__ inline void decode_grad_warp(const GradDecode &p, int prog, unsigned 
     p.flags[prog] = deep ? SR_PF_TOO_DEEP : 0;
     p.nfwd[prog] = deep ? 0 : nf;
     p.nrev[prog] = nr;
-    if (!deep && nf + nr > p.cap_words) *p.big_note = p.tag;
+    if (!deep && nf + nr > p.cap_words) *p.big_note = 1;
   }
 }
 

@@ -152,8 +152,7 @@ struct DecodeArgs {
   int32_t *flags;           // [P] out
   int max_slots;            // stack slots the kernel provides (<= DSM)
   int cap_slots;            // programs that need more than this get NCODE_DEEP (<= max_slots)
-  unsigned long long *ext_note, *deep_note;  // set to `tag` when some program has NCODE_EXT / NCODE_DEEP
-  unsigned long long tag;
+  unsigned long long *ext_note, *deep_note;  // set to 1 when some program has NCODE_EXT / NCODE_DEEP
   // >= 1: a unary operator applied to a variable, u(x_j),
   // reads row xform_row(nvars, u, j) of the variable table instead (the
   // table's first nvars rows are X); with 2, also a base unary operator
