@@ -98,6 +98,11 @@ __device__ __forceinline__ long long next_item(unsigned long long *q, long long 
 __device__ __forceinline__ void launch_wait() {
   asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
 }
+// The same without letting the next kernel in before this one's blocks end: the
+// gradient kernels.  With the merge waiting beside them they took 179 us instead of
+// 165 (2,048 programs x 5,498 cases), 39.3 instead of 36.4 (48 x 512); for the
+// evaluation kernels, whose next is another pass, it makes no difference.
+__device__ __forceinline__ void launch_wait_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... P, typename... A>
 inline cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, int smem, cudaStream_t stream, const A &...args) {
   cudaLaunchConfig_t cfg = {};

@@ -57,7 +57,8 @@ struct GradParams {
   // those, with room for any), [5] the note as that pass reads it (grad_pass);
   // the decode launch zeroes the counters
   unsigned long long *queue;
-  int cap;            // code words per warp of this launch
+  int cap;            // code words that a program of the first pass has at most
+  int room;           // code words per warp of this launch
   int big;            // 1: the big pass
   char *gtape;        // per warp: Lmax entries of GSLOT bytes
   const int32_t *abort;  // sr_set_abort_flag (or NULL)
@@ -69,13 +70,34 @@ struct GradParams {
 __host__ __device__ inline int grad_warp_bytes(int Lmax, int K, int words) {
   return slots_for(Lmax) * GSLOT + 2 * K * 128 + (words * 8 + 15) / 16 * 16;
 }
-// the code words a warp has room for in the main pass: programs of random or
-// evolved populations have at most about 1.9 words a token
-__host__ __device__ inline int grad_cap_words(int Lmax) { return 2 * Lmax + 8; }
+// The code words a warp has room for in the first pass: all that any program can
+// have where they fit beside GMINB CTAs, and then there is no big pass; else 2 a
+// token and a few, or the fewer that one more CTA leaves as long as they are 1.9 a
+// token (most programs of random or evolved populations have less).  With 2 a token
+// and a few whatever the sizes (us): 2,048 programs of <= 24 tokens x 1,637 cases,
+// K = 8, a few of them big, 158 -> 94 (their items come after all others); 512 x
+// 20,000, K = 8, <= 128 tokens 776 -> 733 (3 CTAs -> 4), <= 256 tokens 1,867 -> 1,557
+// (2 -> 3); three Adam steps on 23 problems of <= 16 tokens 311 -> 298 (one launch
+// less a step); the larger share of shared memory costs 1 % on some of 64 tokens.
+constexpr int words_beside(int ctas, int fixed) { return ((233472 / ctas - 1024) / GWARPS / 16 * 16 - fixed) / 8; }
+constexpr int cap_words(int Lmax, int full, int fixed) {
+  if (words_beside(GMINB, fixed) >= full) return full;
+  for (int ctas = GMINB;; --ctas) {
+    const int room = words_beside(ctas, fixed), some = 2 * Lmax + 8;
+    if (10 * room >= 19 * Lmax) return room < some ? room : some;
+  }
+}
+inline int grad_cap_words(int Lmax, int K) {
+  return std::min(grad_code_words(Lmax), cap_words(Lmax, grad_code_words(Lmax), grad_warp_bytes(Lmax, K, 0)));
+}
+static_assert(cap_words(128, 9 * 128 / 2 + 4, 6 * GSLOT + 2 * 8 * 128) == 256, "128 tokens, 8 constants: 4 CTAs");
+static_assert(cap_words(70, 9 * 70 / 2 + 4, 5 * GSLOT + 2 * 8 * 128) == 319, "70 tokens, 8 constants: no big pass");
+// (one CTA leaves the longest programs more than enough: the search ends)
+static_assert(10 * words_beside(1, DSM * GSLOT + 2 * SR_MAX_CONSTS * 128) >= 19 * SR_MAX_LMAX, "cap_words");
 
-__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *queue) {
+__device__ __forceinline__ GradDecode grad_decode_args(const GradParams &p, unsigned long long *queue, int cap) {
   return GradDecode{p.programs, p.lengths, p.consts, p.Lmax, p.K, p.nvars, p.ldx, p.code, p.nfwd, p.nrev, p.flags,
-                    grad_cap_words(p.Lmax), queue + 2};
+                    cap, queue + 2};
 }
 
 // a warp per program
@@ -85,7 +107,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_kernel(GradPara
   if (blockIdx.x == 0 && threadIdx.x < 2) p.queue[threadIdx.x] = 0;
   const int warp = threadIdx.x >> 5, prog = blockIdx.x * DECODE_WARPS + warp;
   if (prog < p.P)
-    decode_grad_warp(grad_decode_args(p, p.queue), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
+    decode_grad_warp(grad_decode_args(p, p.queue, p.cap), prog, dsm + (size_t)warp * grad_scratch_bytes(p.Lmax),
                      slots_for(p.Lmax));
 }
 
@@ -114,9 +136,9 @@ struct GradWarp {
   uint2 *code;
   char *tape;     // this lane's entry of tape entry 0
 };
-__device__ __forceinline__ GradWarp grad_warp(unsigned char *smem, int Lw, int Kw, int cap, char *gtape) {
+__device__ __forceinline__ GradWarp grad_warp(unsigned char *smem, int Lw, int Kw, int room, char *gtape) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char *wb = smem + (size_t)warp * grad_warp_bytes(Lw, Kw, cap);
+  unsigned char *wb = smem + (size_t)warp * grad_warp_bytes(Lw, Kw, room);
   GradWarp w;
   w.slot = (uint32_t)__cvta_generic_to_shared(wb + lane * (GCPL * 4));
   w.sums = reinterpret_cast<float *>(wb + slots_for(Lw) * GSLOT) + lane;
@@ -170,9 +192,9 @@ __device__ __forceinline__ void grad_item(const GradParams &p, int c, int prog, 
 }
 
 // whether a launch takes the program (big: the big pass)
-__device__ __forceinline__ bool grad_takes(const GradParams &p, int prog, int big) {
+__device__ __forceinline__ bool grad_takes(const GradParams &p, int prog, int cap, int big) {
   const int nf = p.nfwd[prog];
-  return nf > 0 && ((nf + p.nrev[prog] > grad_cap_words(p.Lmax)) == (big != 0));
+  return nf > 0 && ((nf + p.nrev[prog] > cap) == (big != 0));
 }
 
 // Whether a pass has programs.  The first hands the decoder's note over to the big
@@ -191,16 +213,16 @@ __device__ __forceinline__ bool grad_pass(unsigned long long *queue, int big) {
 // does not fit the first's share, which returns at once when there are none.
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_kernel(GradParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  launch_wait();
+  launch_wait_only();
   if (!grad_pass(p.queue, p.big)) return;
   const int lane = threadIdx.x & 31;
-  const GradWarp w = grad_warp(smem, p.Lmax, p.K, p.cap, p.gtape);
+  const GradWarp w = grad_warp(smem, p.Lmax, p.K, p.room, p.gtape);
   for (;;) {
     const long long item = next_item(p.queue + p.big, p.total_items, p.abort, p.err, lane);
     if (item >= p.total_items) break;
     const int c = (int)(item / (unsigned long long)p.P);
     const int prog = (int)(item % (unsigned long long)p.P);
-    if (grad_takes(p, prog, p.big)) grad_item(p, c, prog, w, 32 * p.K, lane);
+    if (grad_takes(p, prog, p.cap, p.big)) grad_item(p, c, prog, w, 32 * p.K, lane);
   }
 }
 
@@ -219,7 +241,7 @@ struct GradBatch {
   char *gtape;
   const int32_t *abort;
   unsigned *err;
-  int cap, big;                   // as GradParams
+  int cap, room, big;             // as GradParams
   int Lw, Kw;                     // shared layout: the largest Lmax and K
 };
 
@@ -243,7 +265,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(
   if (g >= b.total_progs) return;
   int q = 0;
   while (q + 1 < b.nprob && b.prog_begin[q + 1] <= g) ++q;
-  decode_grad_warp(grad_decode_args(b.prob[q], b.queue), g - b.prog_begin[q],
+  decode_grad_warp(grad_decode_args(b.prob[q], b.queue, b.cap), g - b.prog_begin[q],
                    dsm + (size_t)warp * grad_scratch_bytes(b.Lw), slots_for(b.prob[q].Lmax));
 }
 
@@ -252,10 +274,10 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) grad_decode_batched_kernel(
 // [item_begin_q, item_begin_q + P_q nchunks_q), chunk-major inside.
 __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_batched_kernel(const __grid_constant__ GradBatch b) {
   extern __shared__ __align__(16) unsigned char smem[];
-  launch_wait();
+  launch_wait_only();
   if (!grad_pass(b.queue, b.big)) return;
   const int lane = threadIdx.x & 31;
-  const GradWarp w = grad_warp(smem, b.Lw, b.Kw, b.cap, b.gtape);
+  const GradWarp w = grad_warp(smem, b.Lw, b.Kw, b.room, b.gtape);
   for (;;) {
     const long long item = next_item(b.queue + b.big, b.total_items, b.abort, b.err, lane);
     if (item >= b.total_items) break;
@@ -263,7 +285,7 @@ __global__ void __launch_bounds__(GWARPS * 32, GMINB) grad_batched_kernel(const 
     const GradParams &p = b.prob[q];
     const long long local = item - b.item_begin[q];
     const int prog = (int)(local % p.P);
-    if (grad_takes(p, prog, b.big)) grad_item(p, (int)(local / p.P), prog, w, 32 * b.Kw, lane);
+    if (grad_takes(p, prog, b.cap, b.big)) grad_item(p, (int)(local / p.P), prog, w, 32 * b.Kw, lane);
   }
 }
 
@@ -373,7 +395,7 @@ sr_status grad_shape(sr_ctx *ctx, int Lw, int Kw, bool batched, GradShape *g) {
   const void *kern = batched ? reinterpret_cast<const void *>(grad_batched_kernel) : reinterpret_cast<const void *>(grad_kernel);
   sr_status st = allow_dynamic_smem(ctx, kern);  // once per (kernel, device): every shape fits
   if (st != SR_OK) return st;
-  g->cap = std::min(grad_cap_words(Lw), grad_code_words(Lw));
+  g->cap = grad_cap_words(Lw, Kw);
   g->big_cap = grad_code_words(Lw) > g->cap ? grad_code_words(Lw) : 0;
   for (int big = 0; big < 2; ++big) {
     int &smem = big ? g->big_smem : g->smem, &grid = big ? g->big_grid : g->grid;
@@ -474,7 +496,7 @@ sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *leng
   gp.gtape = ws + off_t;
   gp.abort = ctx->abort_flag;
   gp.err = ctx->dev_words;
-  gp.cap = gs.cap;
+  gp.cap = gp.room = gs.cap;
   gp.big = 0;
   cudaStream_t s = ctx->stream;
   st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(grad_decode_kernel));
@@ -483,7 +505,7 @@ sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *leng
                             DECODE_WARPS * grad_scratch_bytes(Lmax), s, gp));
   SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.grid, GWARPS * 32, gs.smem, s, gp));
   if (gs.big_cap) {
-    gp.cap = gs.big_cap;
+    gp.room = gs.big_cap;
     gp.big = 1;
     SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.big_grid, GWARPS * 32, gs.big_smem, s, gp));
     ctx->launches += 1;
@@ -571,7 +593,7 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
         p.gtape = nullptr;
         p.abort = nullptr;
         p.err = nullptr;
-        p.cap = 0;
+        p.cap = p.room = 0;
         p.big = 0;
         b->item_begin[g - g0] = items;
         b->prog_begin[g - g0] = progs;
@@ -589,7 +611,7 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
       b->gtape = ctx->ws + off_t;
       b->abort = ctx->abort_flag;
       b->err = ctx->dev_words;
-      b->cap = gs.cap;
+      b->cap = b->room = gs.cap;
       b->big = 0;
       b->Lw = Lw;
       b->Kw = Kw;
@@ -611,7 +633,7 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
                               DECODE_WARPS * 32, DECODE_WARPS * grad_scratch_bytes(Lw), s, b));
     SR_CHECK_CUDA(ctx, launch(grad_batched_kernel, gs.grid, GWARPS * 32, gs.smem, s, b));
     if (gs.big_cap) {
-      b.cap = gs.big_cap;
+      b.room = gs.big_cap;
       b.big = 1;
       SR_CHECK_CUDA(ctx, launch(grad_batched_kernel, gs.big_grid, GWARPS * 32, gs.big_smem, s, b));
       ctx->launches += 1;
