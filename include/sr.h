@@ -446,6 +446,11 @@ sr_status sr_random_programs(sr_ctx *ctx, uint8_t *prog, int32_t *len, float *c,
  * chunks.
  *   arguments as sr_eval; mse device double [P]; dconst device double
  *   [P][K] (K >= 1).  Invalid programs: mse = +inf, dconst = 0.
+ * Workspace: 36 Lmax + 32 bytes of code a program, 256 bytes a program and
+ * case chunk, and a tape of 512 Lmax bytes for each of up to 32 warps per SM.
+ * Where it does not fit and the workspace cannot grow (inside stream capture)
+ * the call runs in slices of the programs that share the room for code, and
+ * on fewer warps: slower, with the same results bit for bit.
  * Errors: SR_EINVAL, SR_ENOMEM, SR_ECUDA.
  */
 sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs,

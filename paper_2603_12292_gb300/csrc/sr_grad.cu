@@ -445,6 +445,89 @@ sr_status check_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *length
   return SR_OK;
 }
 
+// One problem's gradient.  With less room than it would take (as inside stream
+// capture) the programs are decoded and run in slices that share the room for code
+// (4.5 words a token: most of the workspace of a large population), and below a
+// sixteenth of them at a time on fewer blocks (each with its tape).  Slices and
+// blocks do not change a program's items, so results keep their bits.
+sr_status launch_grad(sr_ctx *ctx, const sr_grad_problem &q) {
+  const int P = q.P, Lmax = q.Lmax, K = q.K;
+  GradShape gs;
+  sr_status st = grad_shape(ctx, Lmax, K, false, &gs);
+  if (st != SR_OK) return st;
+  const int chunk = grad_chunk(q.N, (double)grad_chunk_warps(ctx, Lmax, K) * GTARGET_ITEMS_PER_WARP, P);
+  const int nchunks = (q.N + chunk - 1) / chunk;
+  size_t off_q, off_f, off_nc, off_code, off_p, off_t;
+  int per = P, blocks = std::max(gs.grid, gs.big_grid);  // programs of a slice, blocks of a launch
+  for (;;) {
+    Carver cv;
+    off_q = cv.take(256);
+    off_f = cv.take(q.prog_flags ? 0 : (size_t)P * 4);
+    off_nc = cv.take((size_t)per * 8);
+    off_code = cv.take((size_t)per * grad_code_words(Lmax) * 8);
+    off_p = cv.take((size_t)P * nchunks * GSTRIDE * 8);
+    off_t = cv.take((size_t)blocks * GWARPS * Lmax * GSLOT);
+    st = ensure_workspace(ctx, cv.off);
+    if (st != SR_ENOMEM) break;
+    if (per > 1 && (long long)per * 16 > P) per = (per + 1) / 2;
+    else if (blocks > 1) blocks = (blocks + 1) / 2;
+    else break;
+  }
+  if (st != SR_OK) return st;
+  st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(grad_decode_kernel));
+  if (st != SR_OK) return st;
+  char *ws = ctx->ws;
+  double *partials = reinterpret_cast<double *>(ws + off_p);
+  int32_t *flags = q.prog_flags ? q.prog_flags : reinterpret_cast<int32_t *>(ws + off_f);
+  cudaStream_t s = ctx->stream;
+  for (int p0 = 0; p0 < P; p0 += per) {
+    GradParams gp;
+    gp.programs = q.programs + (size_t)p0 * Lmax;
+    gp.lengths = q.lengths + p0;
+    gp.consts = q.consts + (size_t)p0 * K;
+    gp.P = std::min(per, P - p0);
+    gp.Lmax = Lmax;
+    gp.K = K;
+    gp.X = q.X;
+    gp.y = q.y;
+    gp.nvars = q.nvars;
+    gp.N = q.N;
+    gp.ldx = q.ldx;
+    gp.chunk = chunk;
+    gp.nchunks = nchunks;
+    gp.total_items = (long long)gp.P * nchunks;
+    gp.partials = partials + (size_t)p0 * nchunks * GSTRIDE;
+    gp.flags = flags + p0;
+    gp.code = reinterpret_cast<uint2 *>(ws + off_code);
+    gp.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
+    gp.nrev = gp.nfwd + per;
+    gp.queue = reinterpret_cast<unsigned long long *>(ws + off_q);
+    gp.gtape = ws + off_t;
+    gp.abort = ctx->abort_flag;
+    gp.err = ctx->dev_words;
+    gp.cap = gp.room = gs.cap;
+    gp.big = 0;
+    SR_CHECK_CUDA(ctx, launch(grad_decode_kernel, (gp.P + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
+                              DECODE_WARPS * grad_scratch_bytes(Lmax), s, gp));
+    SR_CHECK_CUDA(ctx, launch(grad_kernel, std::min(gs.grid, blocks), GWARPS * 32, gs.smem, s, gp));
+    ctx->launches += 2;
+    if (gs.big_cap) {
+      gp.room = gs.big_cap;
+      gp.big = 1;
+      SR_CHECK_CUDA(ctx, launch(grad_kernel, std::min(gs.big_grid, blocks), GWARPS * 32, gs.big_smem, s, gp));
+      ctx->launches += 1;
+    }
+    SR_CHECK_CUDA(ctx, cudaGetLastError());
+    if (P - p0 <= per) break;  // (p0 + per may be beyond an int)
+  }
+  GradFinal gf{partials, flags, P, q.N, K, nchunks, q.mse, q.dconst};
+  const int per_block = GFINAL_THREADS / grad_final_group(K);
+  SR_CHECK_CUDA(ctx, launch(grad_finalize_kernel, (P + per_block - 1) / per_block, GFINAL_THREADS, 0, s, gf));
+  SR_CHECK_CUDA(ctx, cudaGetLastError());
+  ctx->launches += 1;
+  return SR_OK;
+}
+
 }  // namespace
 }  // namespace sr
 
@@ -458,65 +541,8 @@ sr_status sr_eval_grad(sr_ctx *ctx, const uint8_t *programs, const int32_t *leng
   sr_status st = check_grad(ctx, programs, lengths, consts, P, Lmax, K, X, y, nvars, N, ldx, mse, dconst);
   if (st != SR_OK || P == 0) return st;
   SR_CHECK_CUDA(ctx, cudaSetDevice(ctx->device));
-  GradShape gs;
-  st = grad_shape(ctx, Lmax, K, false, &gs);
-  if (st != SR_OK) return st;
-  const int chunk = grad_chunk(N, (double)grad_chunk_warps(ctx, Lmax, K) * GTARGET_ITEMS_PER_WARP, P);
-  const int nchunks = (N + chunk - 1) / chunk;
-  const long long items = (long long)P * nchunks;
-  Carver cv;
-  const size_t off_q = cv.take(256), off_f = cv.take((size_t)P * 4), off_nc = cv.take((size_t)P * 8),
-               off_code = cv.take((size_t)P * grad_code_words(Lmax) * 8),
-               off_p = cv.take((size_t)items * GSTRIDE * 8),
-               off_t = cv.take((size_t)std::max(gs.grid, gs.big_grid) * GWARPS * Lmax * GSLOT);
-  st = ensure_workspace(ctx, cv.off);
-  if (st != SR_OK) return st;
-  char *ws = ctx->ws;
-  GradParams gp;
-  gp.programs = programs;
-  gp.lengths = lengths;
-  gp.consts = consts;
-  gp.P = P;
-  gp.Lmax = Lmax;
-  gp.K = K;
-  gp.X = X;
-  gp.y = y;
-  gp.nvars = nvars;
-  gp.N = N;
-  gp.ldx = ldx;
-  gp.chunk = chunk;
-  gp.nchunks = nchunks;
-  gp.total_items = items;
-  gp.partials = reinterpret_cast<double *>(ws + off_p);
-  gp.flags = prog_flags ? prog_flags : reinterpret_cast<int32_t *>(ws + off_f);
-  gp.code = reinterpret_cast<uint2 *>(ws + off_code);
-  gp.nfwd = reinterpret_cast<int32_t *>(ws + off_nc);
-  gp.nrev = gp.nfwd + P;
-  gp.queue = reinterpret_cast<unsigned long long *>(ws + off_q);
-  gp.gtape = ws + off_t;
-  gp.abort = ctx->abort_flag;
-  gp.err = ctx->dev_words;
-  gp.cap = gp.room = gs.cap;
-  gp.big = 0;
-  cudaStream_t s = ctx->stream;
-  st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(grad_decode_kernel));
-  if (st != SR_OK) return st;
-  SR_CHECK_CUDA(ctx, launch(grad_decode_kernel, (P + DECODE_WARPS - 1) / DECODE_WARPS, DECODE_WARPS * 32,
-                            DECODE_WARPS * grad_scratch_bytes(Lmax), s, gp));
-  SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.grid, GWARPS * 32, gs.smem, s, gp));
-  if (gs.big_cap) {
-    gp.room = gs.big_cap;
-    gp.big = 1;
-    SR_CHECK_CUDA(ctx, launch(grad_kernel, gs.big_grid, GWARPS * 32, gs.big_smem, s, gp));
-    ctx->launches += 1;
-  }
-  SR_CHECK_CUDA(ctx, cudaGetLastError());
-  GradFinal gf{gp.partials, gp.flags, P, N, K, nchunks, mse, dconst};
-  const int per_block = GFINAL_THREADS / grad_final_group(K);
-  SR_CHECK_CUDA(ctx, launch(grad_finalize_kernel, (P + per_block - 1) / per_block, GFINAL_THREADS, 0, s, gf));
-  SR_CHECK_CUDA(ctx, cudaGetLastError());
-  ctx->launches += 3;
-  return SR_OK;
+  return launch_grad(ctx, sr_grad_problem{programs, lengths, consts, P, Lmax, K, X, y, nvars, N, ldx, mse, dconst,
+                                          prog_flags});
 }
 
 sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob) {
@@ -622,6 +648,11 @@ sr_status sr_eval_grad_batched(sr_ctx *ctx, const sr_grad_problem *pr, int nprob
   for (size_t g0 = 0; g0 < order.size(); g0 += MAX_GBATCH)
     need = std::max(need, group_bytes(g0, std::min(order.size(), g0 + MAX_GBATCH), nullptr));
   st = ensure_workspace(ctx, need);
+  if (st == SR_ENOMEM) {  // with less room one after the other: the same bits, and each may be sliced
+    for (int i : order)
+      if ((st = launch_grad(ctx, pr[i])) != SR_OK) return st;
+    return SR_OK;
+  }
   if (st != SR_OK) return st;
   st = allow_dynamic_smem(ctx, reinterpret_cast<const void *>(grad_decode_batched_kernel));
   if (st != SR_OK) return st;

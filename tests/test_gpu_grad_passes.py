@@ -1,5 +1,6 @@
 """The gradient's second pass, for programs whose code outgrows a warp's share of shared memory: made only where a
-program can be so long, and with the bits of the first pass whichever takes a program."""
+program can be so long, and with the bits of the first pass whichever takes a program.  And its slices, where the
+workspace has no room for the whole call and cannot grow."""
 import numpy as np
 import pytest
 import torch
@@ -42,5 +43,57 @@ def test_the_launch_s_layout_does_not_change_results(ctx):
     batch = sr.sr_eval_grad_batched(ctx, [sr.make_grad_problem(*p) for p in probs])
     sr.sr_sync(ctx)
     for a, b in zip(alone, batch):
+        for u, v in zip(a, b):
+            assert torch.equal(u.view(torch.int64), v.view(torch.int64))
+
+
+def _captured(warm, problems, batched):
+    """The gradients of problems from a call captured on a context whose workspace one call on `warm` has sized, and
+    the kernels it launched."""
+    out = [(torch.empty(p[0].shape[0], dtype=torch.float64, device="cuda"),
+            torch.empty(p[2].shape, dtype=torch.float64, device="cuda")) for p in problems]
+    stream = torch.cuda.Stream()
+    ctx = sr.Context(0, stream)
+    with torch.cuda.stream(stream):
+        sr.sr_eval_grad(ctx, *warm)
+        torch.cuda.synchronize()
+        before = sr.sr_kernel_launches(ctx)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            if batched:
+                sr.sr_eval_grad_batched(ctx, [sr.make_grad_problem(*p, mse=m, dconst=d)
+                                              for p, (m, d) in zip(problems, out)])
+            else:
+                for p, (m, d) in zip(problems, out):
+                    sr.sr_eval_grad(ctx, *p, mse=m, dconst=d)
+        launches = sr.sr_kernel_launches(ctx) - before
+        for _ in range(2):
+            graph.replay()
+    torch.cuda.synchronize()
+    ctx.close()
+    return out, launches
+
+
+def _many(ctx, P, Lmax, K, nvars, N):
+    """P random programs, drawn on the GPU."""
+    prog, lens, c = sr.sr_random_programs(ctx, P, 1, Lmax, K, nvars, -5.0, 5.0, 99, 7)
+    X = torch.rand((nvars, N), device="cuda") * 4 + 1
+    return prog, lens, c, X, torch.sin(X[0]) + X[nvars - 1], N
+
+
+# a workspace sized by 256 programs of 64 tokens holds the tapes but not the code of 40,000; one sized by 4 tokens
+# holds neither the tapes nor the code of 300 programs of 64
+@pytest.mark.parametrize("P,Lmax,warmP,warmL", [(40_000, 64, 256, 64), (300, 64, 256, 4), (1, 64, 1, 1)])
+@pytest.mark.parametrize("batched", [False, True])
+def test_a_captured_call_in_a_small_workspace(ctx, P, Lmax, warmP, warmL, batched):
+    problems = [_many(ctx, P, Lmax, 4, 3, 600)]
+    if batched:
+        problems.append(_many(ctx, 77, 16, 2, 3, 300))
+    want = [sr.sr_eval_grad(ctx, *p) for p in problems]
+    got, launches = _captured(_many(ctx, warmP, warmL, 4, 3, 600), problems, batched)
+    sr.sr_sync(ctx)
+    if P > 10_000:
+        assert launches > 3 * len(problems)
+    for a, b in zip(want, got):
         for u, v in zip(a, b):
             assert torch.equal(u.view(torch.int64), v.view(torch.int64))
