@@ -267,7 +267,7 @@ __device__ inline void decode_eval_warp(const DecodeArgs &p, int prog, unsigned 
   deep = __any_sync(FULL, deep);
   if (lane == 0) {
     p.flags[prog] = deep ? SR_PF_TOO_DEEP : 0;
-    const bool past_cap = used > p.cap_slots;
+    const bool past_cap = used > p.cap_slots || s.cnt[L - 1] >= p.cap_words;
     p.ncode[prog] = deep ? 0 : s.cnt[L - 1] | (ext ? NCODE_EXT : 0) | (past_cap ? NCODE_DEEP : 0);
     if (!deep && ext) *p.ext_note = 1;
     if (!deep && past_cap) *p.deep_note = 1;

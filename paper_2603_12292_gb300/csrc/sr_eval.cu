@@ -102,6 +102,7 @@ struct EvalParams {
   long long ldy;
   int warp_bytes;          // shared memory per warp
   int slots;               // stack slots per warp
+  int words;               // words of code per warp, in the main passes
   int pass;                // Pass: the programs this launch takes
   int score_M;             // Beagle scores: the maximum score per case
   const int32_t *abort;    // sr_set_abort_flag (or NULL)
@@ -114,13 +115,11 @@ struct EvalParams {
   uint8_t *xneed = nullptr;  // the transforms some program reads
 };
 
-// a program's code and its end marker
-__host__ __device__ inline int code_smem_bytes(int Lmax) { return (((Lmax + 1) * 8 + 15) / 16) * 16; }
-
-__host__ __device__ inline int warp_smem_bytes(int slots, int Lmax) {
-  // stack slots | decoded code (8 bytes per token)
-  return slots * SLOT_BYTES + code_smem_bytes(Lmax);
-}
+// shared memory of a warp: stack slots | decoded code, in words of 8 bytes (at most
+// one per token, and the end marker)
+constexpr int code_bytes(int words) { return (words * 8 + 15) / 16 * 16; }
+constexpr int warp_smem_bytes(int slots, int words) { return slots * SLOT_BYTES + code_bytes(words); }
+constexpr int ctas_per_sm(int slots, int words) { return 233472 / (WARPS * warp_smem_bytes(slots, words) + 1024); }
 
 // Stack slots of the main evaluation passes: as many as fit smem_target(minb)
 // beside `code` bytes of code, at most slots_for(Lmax) and at least
@@ -128,18 +127,39 @@ __host__ __device__ inline int warp_smem_bytes(int slots, int Lmax) {
 // rarely need more than 4 (Sethi-Ullman order) while slots_for(256) = 7 would
 // leave room for only 3 CTAs per SM; the few that need more than the main
 // passes give (NCODE_DEEP) run in a third pass with slots_for(Lmax) slots.
-__host__ __device__ inline int fit_slots(int Lmax, int minb, int code) {
+constexpr int fit_slots(int Lmax, int minb, int code) {
   const int full = slots_for(Lmax), lo = full < 4 ? full : 4;
   const int s = (smem_target(minb) / WARPS - code) / SLOT_BYTES;
   return s < lo ? lo : (s > full ? full : s);
 }
-__host__ __device__ inline int shallow_slots(int Lmax, int minb) { return fit_slots(Lmax, minb, code_smem_bytes(Lmax)); }
+// The words of code of the main passes: Lmax + 1, or one less where that saves a
+// CTA per SM (200 and 384 tokens).  Programs that keep an instruction for each of
+// Lmax tokens (none that fuses an operand or folds constants) then run in the third
+// pass too.  2,048 programs x 60,000 cases of <= 200 tokens, 4 CTAs -> 5: 2,524 -> 2,361 us;
+// x 40,000 of <= 384, 3 -> 4: 3,614 -> 3,214.  Where it saves only a slot it gives
+// nothing (256 tokens 3,203 -> 3,197) or costs L1 cache (72 tokens 687 -> 696).
+constexpr int shallow_words(int Lmax, int minb) {
+  const int s = fit_slots(Lmax, minb, code_bytes(Lmax)), t = fit_slots(Lmax, minb, code_bytes(Lmax + 1));
+  const int cs = ctas_per_sm(s, Lmax), ct = ctas_per_sm(t, Lmax + 1);
+  return (cs < minb ? cs : minb) > (ct < minb ? ct : minb) ? Lmax : Lmax + 1;
+}
+constexpr int shallow_slots(int Lmax, int minb) { return fit_slots(Lmax, minb, code_bytes(shallow_words(Lmax, minb))); }
+// shared memory of a CTA in the main passes, and in the third (0: none)
+constexpr int shallow_smem(int Lmax, int minb) {
+  return WARPS * warp_smem_bytes(shallow_slots(Lmax, minb), shallow_words(Lmax, minb));
+}
+constexpr int deep_smem(int Lmax, int minb) {
+  return slots_for(Lmax) > shallow_slots(Lmax, minb) || shallow_words(Lmax, minb) <= Lmax
+             ? WARPS * warp_smem_bytes(slots_for(Lmax), Lmax + 1)
+             : 0;
+}
+
 
 // 5 CTAs per SM where they fit with at least min(slots_for(Lmax), 4) slots
-// (Lmax <= 198), else 4.
-inline int minb_for(int Lmax) {
-  return WARPS * warp_smem_bytes(shallow_slots(Lmax, 5), Lmax) <= smem_target(5) ? 5 : 4;
-}
+// (Lmax <= 200), else 4.
+constexpr int minb_for(int Lmax) { return shallow_smem(Lmax, 5) <= smem_target(5) ? 5 : 4; }
+static_assert(minb_for(200) == 5 && minb_for(201) == 4, "5 CTAs per SM up to 200 tokens");
+static_assert(shallow_smem(384, 4) <= smem_target(4), "384 tokens: 4 CTAs per SM");
 // The evaluation's CTAs per SM: the tuned choice where it fits, else the
 // automatic one
 inline int eval_minb(int Lmax, int tuned) {
@@ -257,8 +277,8 @@ __device__ void ycenter_chunk(const float *y, int N, int chunk, int nchunks, int
 
 
 // ---------------------------------------------------------------- decode pre-pass
-// cap_slots: programs that need more get NCODE_DEEP
-__device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_slots) {
+// slots, words: those of the main passes; programs that need more get NCODE_DEEP
+__device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int slots, int words) {
   DecodeArgs a;
   a.programs = p.programs;
   a.lengths = p.lengths;
@@ -272,7 +292,8 @@ __device__ __forceinline__ DecodeArgs decode_args(const EvalParams &p, int cap_s
   a.ncode = p.ncode;
   a.flags = p.flags;
   a.max_slots = slots_for(p.Lmax);
-  a.cap_slots = cap_slots;
+  a.cap_slots = slots;
+  a.cap_words = words;
   a.ext_note = p.queue + 2;
   a.deep_note = p.queue + 4;
   a.xform = p.xform;
@@ -314,7 +335,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_kernel(EvalParams p)
   }
   const int warp = threadIdx.x >> 5, prog = block * DECODE_WARPS + warp;
   if (prog < p.P)
-    decode_eval_warp(decode_args(p, p.slots), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
+    decode_eval_warp(decode_args(p, p.slots, p.words), prog, dsm + (size_t)warp * decode_scratch_bytes(p.Lmax));
 }
 
 // The variable table of an evaluation with transforms (DecodeArgs::xform):
@@ -670,8 +691,8 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
 // Up to three passes over the work items: the programs of the base operators
 // (and the invalid ones), those that use 1/x, tan, asin, acos, atan or tanh
 // (which returns at once when there are none), and those that need
-// more than the main passes' shallow_slots(Lmax, MINB) stack slots (NCODE_DEEP;
-// made only when slots_for(Lmax) is more).  Keeping the extended operators out
+// more than the main passes' shallow_slots(Lmax, MINB) stack slots or shallow_words
+// (NCODE_DEEP; made only where a program can).  Keeping the extended operators out
 // of the first kernel keeps its loop inside the instruction cache.  Where the
 // rows of X could not be laid out for 256-bit loads, one pass of the EXT kernel
 // without them takes the base and the extended programs.
@@ -757,7 +778,7 @@ struct BatchParams {
   long long total_items;
   unsigned long long *queue;  // as EvalParams::queue
   int warp_bytes;
-  int slots;
+  int slots, words;           // as EvalParams
   int maxL;                   // the largest Lmax of the batch
   int pass;                   // as EvalParams::pass
   // blocks of the decode launch: those that sum chunks of y, that decode, that copy X
@@ -834,7 +855,7 @@ __global__ void __launch_bounds__(DECODE_WARPS * 32) decode_batched_kernel(const
   }
   EvalParams p = view(b.prob[lo]);
   p.queue = b.queue;
-  decode_eval_warp(decode_args(p, b.slots), g - b.prob[lo].prog_begin,
+  decode_eval_warp(decode_args(p, b.slots, b.words), g - b.prob[lo].prog_begin,
                    dsm + (size_t)warp * decode_scratch_bytes(b.maxL));
 }
 
@@ -1136,7 +1157,7 @@ sr_status launch_pass(sr_ctx *ctx, int mode, bool ext, bool wide, int minb, int 
 
 struct Plan {
   int minb;       // CTAs per SM of the main passes (eval_kernel's MINB)
-  int slots;      // stack slots per warp of the main passes
+  int slots, words;  // stack slots and words of code per warp of the main passes
   int smem, chunk, nchunks;
   int smem_deep;  // shared memory of the deep pass (0: none)
   long long items;
@@ -1172,8 +1193,9 @@ enum Layout { LAY_TABLE, LAY_COPY, LAY_PLAIN };
 void make_plan(sr_ctx *ctx, int P, int Lmax, int N, Plan *pl, int nvars, bool x_wide, Layout lay) {
   pl->minb = eval_minb(Lmax, ctx->eval_ctas);
   pl->slots = shallow_slots(Lmax, pl->minb);
-  pl->smem = WARPS * warp_smem_bytes(pl->slots, Lmax);
-  pl->smem_deep = slots_for(Lmax) > pl->slots ? WARPS * warp_smem_bytes(slots_for(Lmax), Lmax) : 0;
+  pl->words = shallow_words(Lmax, pl->minb);
+  pl->smem = shallow_smem(Lmax, pl->minb);
+  pl->smem_deep = deep_smem(Lmax, pl->minb);
   const long long warps =
       (long long)chunk_ctas(Lmax, chunk_minb(Lmax, ctx->eval_ctas)) * ctx->num_sms * WARPS;
   const long long want = warps * TARGET_ITEMS_PER_WARP;
@@ -1286,7 +1308,8 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   ep.yhat = yhat;
   ep.ldy = ldy;
   ep.slots = pl.slots;
-  ep.warp_bytes = warp_smem_bytes(pl.slots, Lmax);
+  ep.words = pl.words;
+  ep.warp_bytes = pl.smem / WARPS;
   ep.pass = PASS_BASE;
   ep.abort = ctx->abort_flag;
   ep.err = ctx->dev_words;
@@ -1332,7 +1355,7 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
   if (st == SR_OK && pl.smem_deep) {
     ep.pass = PASS_DEEP;
     ep.slots = slots_for(Lmax);
-    ep.warp_bytes = warp_smem_bytes(ep.slots, Lmax);
+    ep.warp_bytes = pl.smem_deep / WARPS;
     st = launch_pass(ctx, mode, true, pl.wide, 4, pl.smem_deep, ep);
   }
   if (st != SR_OK) return st;
@@ -1389,10 +1412,8 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
   // and registers, 5 more warps); it must leave room for min(slots_for, 4)
   // stack slots
   int bminb = ctx->batched_ctas ? ctx->batched_ctas : 4;
-  if (bminb == 5 && WARPS * warp_smem_bytes(shallow_slots(maxL, 5), maxL) > smem_target(5)) bminb = 4;
-  const int bslots = shallow_slots(maxL, bminb);
-  const int smem = WARPS * warp_smem_bytes(bslots, maxL);
-  const int smem_deep = slots_for(maxL) > bslots ? WARPS * warp_smem_bytes(slots_for(maxL), maxL) : 0;
+  if (bminb == 5 && shallow_smem(maxL, 5) > smem_target(5)) bminb = 4;
+  const int smem = shallow_smem(maxL, bminb), smem_deep = deep_smem(maxL, bminb);
   // the cases per item by chunk_ctas' rule, whatever the kernels take
   const int code = ((maxL * 8 + 15) / 16) * 16;
   const int cminb = ctx->batched_ctas == 5 && WARPS * (fit_slots(maxL, 5, code) * SLOT_BYTES + code) > smem_target(5)
@@ -1526,9 +1547,10 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       bpar->total_progs = progs;
       bpar->total_items = items;
       bpar->queue = reinterpret_cast<unsigned long long *>(ctx->ws + off_q);
-      bpar->slots = bslots;
+      bpar->slots = shallow_slots(maxL, bminb);
+      bpar->words = shallow_words(maxL, bminb);
       bpar->maxL = maxL;
-      bpar->warp_bytes = warp_smem_bytes(bpar->slots, maxL);
+      bpar->warp_bytes = smem / WARPS;
       bpar->pass = PASS_BASE;
       bpar->decode_blocks = (progs + DECODE_WARPS - 1) / DECODE_WARPS;
       bpar->stage_blocks = stages;
@@ -1591,7 +1613,7 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       BatchParams bd = b;
       bd.pass = PASS_DEEP;
       bd.slots = slots_for(maxL);
-      bd.warp_bytes = warp_smem_bytes(bd.slots, maxL);
+      bd.warp_bytes = smem_deep / WARPS;
       st = launch_batch_pass(ctx, true, wide, 4, smem_deep, bd);
     }
     if (st != SR_OK) return st;

@@ -23,7 +23,7 @@ static_assert(SR_MAX_LMAX <= 512, "8 slots cover programs of up to 512 tokens");
 // The slots programs of up to Lmax tokens can need: floor(log2(leaves)) with
 // leaves <= (Lmax + 1) / 2.  Kernels size their shared stack by it (6 slots
 // for Lmax = 128 instead of 8 -- more warps per SM).
-__host__ __device__ inline int slots_for(int Lmax) {
+__host__ __device__ constexpr int slots_for(int Lmax) {
   int leaves = (Lmax + 1) / 2, s = 0;
   while ((2 << s) <= leaves) ++s;
   return s < 1 ? 1 : (s > DSM ? DSM : s);
@@ -133,8 +133,9 @@ enum Op : uint32_t {
 // keep the loop of the base operators free of the extra call site.
 constexpr int NCODE_EXT = 1 << 30;
 // NCODE_DEEP is set when the program needs more stack slots than the
-// decoder's cap_slots: the evaluation kernels give most programs a few slots
-// (more warps fit on an SM) and run the rare deeper ones in a separate pass.
+// decoder's cap_slots (or more words than its cap_words): the evaluation kernels
+// give most programs a few slots (more warps fit on an SM) and run the rare deeper
+// ones in a separate pass.
 constexpr int NCODE_DEEP = 1 << 29;
 __device__ __forceinline__ int ncode_count(int v) { return v & 0xffff; }
 __device__ __forceinline__ bool ncode_ext(int v) { return (v & NCODE_EXT) != 0; }
@@ -151,7 +152,8 @@ struct DecodeArgs {
   int32_t *ncode;           // [P] out
   int32_t *flags;           // [P] out
   int max_slots;            // stack slots the kernel provides (<= DSM)
-  int cap_slots;            // programs that need more than this get NCODE_DEEP (<= max_slots)
+  int cap_slots;            // programs that need more than this get NCODE_DEEP (<= max_slots),
+  int cap_words;            // and so do those with more words than this, their end marker counted
   unsigned long long *ext_note, *deep_note;  // set to 1 when some program has NCODE_EXT / NCODE_DEEP
   // >= 1: a unary operator applied to a variable, u(x_j),
   // reads row xform_row(nvars, u, j) of the variable table instead (the
