@@ -623,7 +623,7 @@ __device__ __forceinline__ V4 div4(const V4 &a, const V4 &b) {  // the protected
   unpack4(b, y);
   bool ok = true;
 #pragma unroll
-  for (int i = 0; i < GCPL; ++i) ok = ok & (fabsf(y[i]) <= 8.5e37f);
+  for (int i = 0; i < GCPL; ++i) ok = ok & (fabsf(y[i]) <= DIV_NEAR);
   if (__any_sync(FULL, !ok)) return div4_wide(a, b);
 #pragma unroll
   for (int i = 0; i < GCPL; ++i) x[i] = DivNear()(x[i], y[i]);

@@ -34,10 +34,8 @@ __host__ __device__ constexpr int slots_for(int Lmax) {
 // full range, at most 2 ulp off (subnormal results included) -- within the
 // 2-ulp allowance the oracle's enclosure gives every operation.  Computed
 // whatever b is and selected, so the vector loops stay branch-free.
-// Measured on the paper-shaped population: +12 % over the IEEE quotient,
-// whose longer sequence also pushed the interpreter loop out of the
-// instruction cache; a redo of the subnormal results by the IEEE quotient
-// cost back 11 %.
+// Measured on the paper-shaped population: +12 % over the IEEE quotient; a redo of
+// the subnormal results by the IEEE quotient cost back 11 %.
 __device__ __forceinline__ float op_div(float a, float b) {
   float q;
   asm("div.full.f32 %0, %1, %2;" : "=f"(q) : "f"(a), "f"(b));
