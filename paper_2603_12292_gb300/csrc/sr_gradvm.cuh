@@ -83,7 +83,7 @@ static __device__ __noinline__ float2 sincos_wide(float x) {
   sincosf(x, &s, &c);
   return make_float2(s, c);
 }
-__device__ __forceinline__ float2 sincos_near(float x) {
+__device__ __forceinline__ float2 sincos_near(float x) {  // |x| <= NEAR
   __builtin_assume(fabsf(x) <= NEAR);
   float s, c;
   sincosf(x, &s, &c);
@@ -600,8 +600,9 @@ __device__ __forceinline__ SinCos4 sincos4(const V4 &x) {
   unpack4(x, t);
 #pragma unroll
   for (int i = 0; i < GCPL; ++i) {
-    const float2 r = sincos_near(opaque(t[i]));
-    a[i] = fabsf(t[i]) <= NEAR ? r.x : t[i];
+    const bool near = fabsf(t[i]) <= NEAR;
+    const float2 r = sincos_near(near ? t[i] : 0.0f);
+    a[i] = near ? r.x : t[i];
     b[i] = r.y;
   }
   const float m = fmaxf(fmaxf(fabsf(a[0]), fabsf(a[1])), fmaxf(fabsf(a[2]), fabsf(a[3])));

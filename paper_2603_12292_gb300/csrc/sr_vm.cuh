@@ -102,31 +102,30 @@ __device__ __forceinline__ V8 zip8(const V8 &a, const V8 &b, F f) {
   return pack8(t);
 }
 
-// sin and cos: the library's path for moderate arguments runs on every value;
-// an argument outside it (|x| > 4e4) is passed through instead of its result and
-// recognised afterwards by its magnitude (a result is at most 1), for the whole
-// warp at once: one test instead of a branch per value.  The argument of the
-// library call is hidden from the optimiser, which would otherwise conclude from
-// its range that no value is ever outside.
-__device__ __forceinline__ float opaque(float x) {
-  asm("" : "+f"(x));
-  return x;
-}
+// sin and cos: the library's path for moderate arguments runs on every value; an
+// argument outside it (|x| > 4e4, or NaN) is replaced by 0 for that, passed through
+// instead of the result and recognised afterwards by its magnitude (a result is at
+// most 1), for the whole warp at once: one test instead of a branch per value.  The 0
+// makes the assumption true for every value that it is stated of; assumed of the
+// arguments as they are, though used for the moderate ones only, 8,192 x 131,072 took
+// 25.2 ms instead of 25.4, 1,500 x 100,003 2,043 us instead of 2,066.
 constexpr float NEAR = 4.0e4f;
 struct SinNear {
   __device__ __forceinline__ float operator()(float x) const {
-    const float xn = opaque(x);
+    const bool near = fabsf(x) <= NEAR;
+    const float xn = near ? x : 0.0f;
     __builtin_assume(fabsf(xn) <= NEAR);
     const float r = sinf(xn);
-    return fabsf(x) <= NEAR ? r : x;
+    return near ? r : x;
   }
 };
 struct CosNear {
   __device__ __forceinline__ float operator()(float x) const {
-    const float xn = opaque(x);
+    const bool near = fabsf(x) <= NEAR;
+    const float xn = near ? x : 0.0f;
     __builtin_assume(fabsf(xn) <= NEAR);
     const float r = cosf(xn);
-    return fabsf(x) <= NEAR ? r : x;
+    return near ? r : x;
   }
 };
 struct SinFar { __device__ __forceinline__ float operator()(float x) const { return fabsf(x) > 2.0f ? sin_wide(x) : x; } };
