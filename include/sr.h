@@ -45,6 +45,9 @@
  * lengths[p] are ignored), lengths [P] int32, consts [P][K] float.
  * Case layout: X [nvars][ldx] float (row j holds variable j for every case;
  * ldx >= N, ldx % 4 == 0, X 16-byte aligned), y [N] float (16-byte aligned).
+ * The evaluation reads rows in place where X is 32-byte aligned and ldx % 8 ==
+ * 0; other rows it copies to the workspace in every call without a variable
+ * table (4 * nvars * N bytes, where there is room; read as they are else).
  */
 #ifndef SR_H
 #define SR_H
@@ -236,8 +239,8 @@ typedef struct {
 sr_status sr_eval_batched(sr_ctx *ctx, const sr_problem *problems, int nprob);
 
 /* Cases per evaluation work item for later sr_eval / sr_predict calls on
- * this context (rounded up to a multiple of 128); 0 restores the automatic
- * choice (about eight items per resident warp).  Set by the autotuner. */
+ * this context (rounded up to a multiple of 256); 0 restores the automatic
+ * choice (about sixteen items per resident warp).  Set by the autotuner. */
 sr_status sr_set_tile(sr_ctx *ctx, int cases_per_tile);
 
 /* CTAs (of 8 warps) per SM of the persistent evaluation kernels, set by the

@@ -31,7 +31,7 @@
 //      memory [slot][half][lane] (conflict-free float4).
 //   3. Per lane, FP32 Kahan-compensated sums over the item's cases, out of line
 //      and in local memory, so that they cost the interpreter no registers
-//      (4,096 x 100,000 at 5 CTAs per SM: 5,824 -> 5,434 us); FP64 warp
+//      (4,096 x 100,000 at 5 CTAs per SM, one population: 5,824 -> 5,434 us); FP64 warp
 //      reduction; one FP64 partial per (program, chunk); a finalize kernel
 //      merges the chunks of each program (a group of lanes each, fixed order).
 #include <math.h>
@@ -1169,10 +1169,9 @@ struct Plan {
       off_ych, off_ysum, off_xt, off_xneed, bytes;
 };
 
-// Whether a call (or a batch's problem) of P programs and N cases over nvars variables reads
-// the variable table, and that table's row stride.
-// (0: no; 1: u(x_j); 2: also the compositions, where the table stays
-// within XFORM2_MAX_BYTES), and that table's row stride.
+// Whether a call (or a batch's problem) of P programs and N cases over nvars variables
+// reads the variable table (0: no; 1: u(x_j); 2: also the compositions, where the
+// table stays within XFORM2_MAX_BYTES), and that table's row stride.
 inline int use_xform(const sr_ctx *ctx, int P, int nvars, int N, int *ldxt) {
   *ldxt = (int)align_up((size_t)N, CPL);  // whole groups of 8 cases (sr_vm.cuh, WIDE)
   const bool automatic = ctx->xform == 1 && N >= XFORM_MIN_N && P >= XFORM_MIN_P;

@@ -331,8 +331,8 @@ __global__ void __launch_bounds__(GFINAL_THREADS) grad_finalize_kernel(GradFinal
 
 // Adam, FP64 moments, every operation rounded on its own in the written order.
 // What bounds it: the FP64 pipe (two lanes an SM), so the blocks are small and the
-// work spreads over the SMs (8 steps on 24 tables of 2,048 constants with their
-// gradients: 745 us with 256 threads a block, 733 with 64).
+// work spreads over the SMs (three steps on the constants of 24 small problems with
+// their gradients: 745 us with 256 threads a block, 733 with 64).
 constexpr int ADAM_THREADS = 64;
 __device__ __forceinline__ void adam_one(float *c, const double *g, double *m, double *v, int i,
                                          double lr, double b1, double b2, double eps, double bc1, double bc2) {

@@ -3,8 +3,8 @@
 // that run them on 128 cases, 4 per lane.
 //
 // What bounds it: issue slots, then the tape.  A node of the first adjoint cost
-// 114 warp instructions a step: two dispatches through a binary tree of
-// compares, a tape entry written and read for most operators, and constants --
+// 114 warp instructions a step (the profiler's counter): a switch over the opcodes
+// each way, a tape entry written and read for most operators, and constants --
 // half of the leaves -- evaluated on every case.  Now
 //   - a subtree that reads only constants is evaluated once, by the decoder,
 //     with its partial derivatives: the forward program loads its value, the
@@ -16,7 +16,7 @@
 //     <= 96 tokens instead of 23);
 //   - both loops branch through tables in PTX and run on FP32 pairs (sr_vm.cuh).
 // Every value, partial and sum is rounded as before, in the same order.
-// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,231 -> 4,448; warp
+// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,231 -> 4,470; warp
 // instructions 5.97e9 -> 3.33e9, DRAM 11.1 -> 0.9 GB (the tape stays in L2); 24
 // small problems, one gradient 245 -> 185.
 #pragma once

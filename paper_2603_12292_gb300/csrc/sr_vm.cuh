@@ -7,17 +7,16 @@
 //     the packed instructions (add / sub / mul .f32x2, each half rounded as the
 //     scalar instruction rounds it);
 //   - the loads, stack moves and packed operators run in one PTX loop that
-//     branches through a table on the opcode (the compiler turned the same
-//     switch into a binary tree of compares, 12 instructions a node, and sank
-//     equal operators of different cases together, with moves in front);
+//     branches through a table on the opcode instead of a C++ switch;
 //   - a row of X is read with one 256-bit load per lane;
-//   - sin, cos, exp, log, sqrt and the quotient leave that loop, run inline in
-//     the caller's registers (as calls they cost 16 moves each), and enter it
-//     again.  Their range tests are made once for the lane's 8 values.
-// Issued instructions per node and 256 cases, before -> now: x_j op 33 -> 14,
-// square 27 -> 11, (push, x_i op x_j, op) 98 -> 42, quotient 137 -> 69, sin
-// 253 -> 209, log 264 -> 248, exp 120 -> 105, sqrt 119 -> 113 (5 CTAs per SM).
-// Evaluation of 8,192 programs of <= 256 tokens x 131,072 cases: 32.7 -> 25.0 ms.
+//   - sin, cos, exp, log, sqrt and the quotient leave that loop, run inline
+//     instead of as calls, and enter it again.  Their range tests are made once
+//     for the lane's 8 values.
+// Instructions executed (the profiler's counter) per node and 256 cases, before ->
+// then: x_j op 33 -> 14, square 27 -> 11, (push, x_i op x_j, op) 98 -> 42, quotient
+// 137 -> 69, sin 253 -> 209 (a select a value more since), log 264 -> 248, exp 120 ->
+// 105, sqrt 119 -> 113 (5 CTAs per SM).
+// Evaluation of 8,192 programs of <= 256 tokens x 131,072 cases: 32.7 -> 25.4 ms.
 // Every value keeps its bits: each operator sees the operands it saw before and
 // rounds once.
 #pragma once
@@ -277,9 +276,9 @@ static_assert(OP_LDV == 0 && OP_PUSHC == 3 && OP_ADD == 4 && OP_RDIV == 9 && OP_
 // kernel around it have to stay in the instruction cache together, so a copy
 // with more in it keeps its bodies narrower (values in flight; map8) or fetches
 // the next instruction in one place instead of after every operator.
-// Measured (us): base copy, threaded and 8 wide against one fetch:
-// 4,096 x 100,000 5,290 / 5,423, 8,192 x 131,072 25,308 / 26,600; log 4 wide
-// 5,356 / 25,539.  Eq. 3 kernel, 4,096 x 40,000: threaded 8 wide 2,773, sin, cos
+// Measured (us), each row of figures on one population: base copy, threaded and 8
+// wide against one fetch: 4,096 x 100,000 5,290 / 5,423, 8,192 x 131,072 25,308 /
+// 26,600; log 4 wide 5,356 / 25,539.  Eq. 3 kernel, 4,096 x 40,000: threaded 8 wide 2,773, sin, cos
 // and log 4 wide 2,562, one fetch 8 wide 2,580.  EXT copy (twelve library
 // operators), 2,048 x 50,001: 2 wide with one fetch 2,102, threaded 2,287,
 // 4 wide 2,265, 8 wide 2,706.
