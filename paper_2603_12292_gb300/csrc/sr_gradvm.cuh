@@ -579,7 +579,14 @@ static_assert(FW_TAPE == 16 && FW_SQT == 19 && FW_DIV == 20 && FW_CRDIV == 25 &&
 struct SinCos4 {
   V4 s, c;
 };
-// an argument beyond the library's moderate range (any_far's way, sr_vm.cuh)
+// the larger value, NaN if either is
+__device__ __forceinline__ float max_nan(float a, float b) {
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(a) : "f"(b));
+  return a;
+}
+// arguments beyond the library's moderate range (any_far's way, sr_vm.cuh), and NaN,
+// whose cosine is that of the 0 it was replaced by until here.  With a select per
+// value for it in sincos4, 2,048 x 65,536 took 4,529 us instead of 4,496.
 __device__ __noinline__ SinCos4 sincos4_far(V4 s, V4 c) {
   float a[GCPL], b[GCPL];
   unpack4(s, a);
@@ -588,6 +595,7 @@ __device__ __noinline__ SinCos4 sincos4_far(V4 s, V4 c) {
   for (int i = 0; i < GCPL; ++i) {
     float2 r = make_float2(a[0], b[0]);
     if (fabsf(r.x) > 2.0f) r = sincos_wide(r.x);
+    else if (r.x != r.x) r.y = r.x;
 #pragma unroll
     for (int j = 0; j < GCPL - 1; ++j) a[j] = a[j + 1], b[j] = b[j + 1];
     a[GCPL - 1] = r.x;
@@ -605,9 +613,9 @@ __device__ __forceinline__ SinCos4 sincos4(const V4 &x) {
     a[i] = near ? r.x : t[i];
     b[i] = r.y;
   }
-  const float m = fmaxf(fmaxf(fabsf(a[0]), fabsf(a[1])), fmaxf(fabsf(a[2]), fabsf(a[3])));
+  const float m = max_nan(max_nan(fabsf(a[0]), fabsf(a[1])), max_nan(fabsf(a[2]), fabsf(a[3])));
   SinCos4 r{pack4(a), pack4(b)};
-  if (__any_sync(FULL, m > 2.0f)) r = sincos4_far(r.s, r.c);
+  if (__any_sync(FULL, !(m <= 2.0f))) r = sincos4_far(r.s, r.c);
   return r;
 }
 __device__ __noinline__ V4 div4_wide(V4 a, V4 b) {
