@@ -694,16 +694,18 @@ __device__ __forceinline__ void eval_item(const EvalParams &p, int c, int prog, 
 // more than the main passes' shallow_slots(Lmax, MINB) stack slots or shallow_words
 // (NCODE_DEEP; made only where a program can).  Keeping the extended operators out
 // of the first kernel keeps its loop inside the instruction cache.  Where the
-// rows of X could not be laid out for 256-bit loads, one pass of the EXT kernel
-// without them takes the base and the extended programs.
-enum Pass { PASS_BASE = 0, PASS_EXT = 1, PASS_DEEP = 2, PASS_SHALLOW = 3 };
+// rows of X could not be laid out for 256-bit loads, the same passes read them in
+// halves.  (One pass of the EXT kernel for base and extended programs then took,
+// 1,500 programs of <= 64 tokens x 500,004 cases, 7,535 us instead of 6,105; 1,024 of
+// <= 128 x 400,004, both kinds, 7,810 instead of 6,260.)
+enum Pass { PASS_BASE = 0, PASS_EXT = 1, PASS_DEEP = 2 };
 
 __device__ __forceinline__ bool takes(int pass, int ncode) {
   if (pass == PASS_DEEP) return ncode_deep(ncode);
   if (ncode_deep(ncode)) return false;
-  return pass == PASS_SHALLOW || ncode_ext(ncode) == (pass == PASS_EXT);
+  return ncode_ext(ncode) == (pass == PASS_EXT);
 }
-// The first pass (base or shallow) hands the decoder's notes over to the passes
+// The first pass hands the decoder's notes over to the passes
 // after it and clears them for the next call.  A replay of a captured call then
 // makes a pass only when its own programs need it (a note that stayed had every
 // replay after it walk the items of an empty pass).
@@ -1114,11 +1116,12 @@ __global__ void __launch_bounds__(FINAL_THREADS) finalize_batched_kernel(const _
 // ---------------------------------------------------------------- host side
 typedef void (*EvalKernel)(EvalParams);
 
-// The instantiations: base and EXT with 4 or 5 CTAs per SM, and the EXT one
-// that reads rows in halves (4 CTAs).
+// The instantiations: base and EXT with 4 or 5 CTAs per SM, and those that read
+// rows in halves (4 CTAs the EXT one).
 template <int MODE>
 EvalKernel eval_kernel_m(bool ext, bool wide, int minb) {
-  if (!wide) return eval_kernel<MODE, true, false, 4>;
+  if (!wide && ext) return eval_kernel<MODE, true, false, 4>;
+  if (!wide) return minb == 5 ? eval_kernel<MODE, false, false, 5> : eval_kernel<MODE, false, false, 4>;
   if (minb == 5) return ext ? eval_kernel<MODE, true, true, 5> : eval_kernel<MODE, false, true, 5>;
   return ext ? eval_kernel<MODE, true, true, 4> : eval_kernel<MODE, false, true, 4>;
 }
@@ -1343,14 +1346,9 @@ sr_status launch_eval(sr_ctx *ctx, int mode, const uint8_t *programs, const int3
     SR_CHECK_CUDA(ctx, launch(ycenter_kernel, pl.nchunks, PREP_THREADS, 0, s, cp));
     ctx->launches += 1;
   }
-  if (pl.wide) {
-    st = launch_pass(ctx, mode, false, true, pl.minb, pl.smem, ep);
-    ep.pass = PASS_EXT;
-    if (st == SR_OK) st = launch_pass(ctx, mode, true, true, pl.minb, pl.smem, ep);
-  } else {
-    ep.pass = PASS_SHALLOW;
-    st = launch_pass(ctx, mode, true, false, 4, pl.smem, ep);
-  }
+  st = launch_pass(ctx, mode, false, pl.wide, pl.minb, pl.smem, ep);
+  ep.pass = PASS_EXT;
+  if (st == SR_OK) st = launch_pass(ctx, mode, true, pl.wide, pl.minb, pl.smem, ep);
   if (st == SR_OK && pl.smem_deep) {
     ep.pass = PASS_DEEP;
     ep.slots = slots_for(Lmax);
@@ -1377,7 +1375,7 @@ BatchKernel batch_kernel_m(bool ext, bool lean) {
   return lean ? eval_batched_kernel<false, true, MINB, true> : eval_batched_kernel<false, true, MINB, false>;
 }
 BatchKernel batch_kernel_for(bool ext, bool wide, int minb, bool lean) {
-  if (!wide) return eval_batched_kernel<true, false, 4, false>;
+  if (!wide) return ext ? eval_batched_kernel<true, false, 4, false> : eval_batched_kernel<false, false, 4, false>;
   return minb == 3 ? batch_kernel_m<3>(ext, lean) : (minb == 5 ? batch_kernel_m<5>(ext, lean) : batch_kernel_m<4>(ext, lean));
 }
 sr_status launch_batch_pass(sr_ctx *ctx, bool ext, bool wide, int minb, int smem, const BatchParams &b, bool lean = false) {
@@ -1598,16 +1596,11 @@ sr_status launch_batched(sr_ctx *ctx, const sr_problem *pr, int nprob) {
       SR_CHECK_CUDA(ctx, launch(ycenter_batched_kernel, b.ysum_blocks, PREP_THREADS, 0, s, b));
       ctx->launches += 1;
     }
-    if (wide) {
-      double steps = 0.0;
-      for (int r = 0; r < b.nprob; ++r) steps += (double)b.prob[r].P * ((b.prob[r].N + STEP - 1) / STEP);
-      st = launch_batch_pass(ctx, false, true, bminb, smem, b, steps <= (double)LEAN_MAX_STEPS * (double)b.total_items);
-      b.pass = PASS_EXT;
-      if (st == SR_OK) st = launch_batch_pass(ctx, true, true, bminb, smem, b);
-    } else {
-      b.pass = PASS_SHALLOW;
-      st = launch_batch_pass(ctx, true, false, 4, smem, b);
-    }
+    double steps = 0.0;
+    for (int r = 0; r < b.nprob; ++r) steps += (double)b.prob[r].P * ((b.prob[r].N + STEP - 1) / STEP);
+    st = launch_batch_pass(ctx, false, wide, bminb, smem, b, steps <= (double)LEAN_MAX_STEPS * (double)b.total_items);
+    b.pass = PASS_EXT;
+    if (st == SR_OK) st = launch_batch_pass(ctx, true, wide, bminb, smem, b);
     if (st == SR_OK && smem_deep) {
       BatchParams bd = b;
       bd.pass = PASS_DEEP;

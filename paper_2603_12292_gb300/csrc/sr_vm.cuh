@@ -311,6 +311,9 @@ __device__ __forceinline__ V8 interpret(const uint2 *code, const char *stk, cons
       asm volatile(SR_CORE(SR_LDX_WIDE, SR_LDT_WIDE, SR_FETCH) : SR_CORE_OUT(T, X, ip, op) : "r"(st), "l"(xa) : "memory");
     else if (WIDE)
       asm volatile(SR_CORE(SR_LDX_WIDE, SR_LDT_WIDE, SR_JUMP) : SR_CORE_OUT(T, X, ip, op) : "r"(st), "l"(xa) : "memory");
+    else if (S::THREADED)
+      asm volatile(SR_CORE(SR_LDX_HALVES, SR_LDT_HALVES, SR_FETCH)
+                   : SR_CORE_OUT(T, X, ip, op) : "r"(st), "l"(xa), "l"(xb) : "memory");
     else
       asm volatile(SR_CORE(SR_LDX_HALVES, SR_LDT_HALVES, SR_JUMP)
                    : SR_CORE_OUT(T, X, ip, op) : "r"(st), "l"(xa), "l"(xb) : "memory");
