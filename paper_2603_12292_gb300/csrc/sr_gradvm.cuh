@@ -16,7 +16,7 @@
 //     <= 96 tokens instead of 23);
 //   - both loops branch through tables in PTX and run on FP32 pairs (sr_vm.cuh).
 // Every value, partial and sum is rounded as before, in the same order.
-// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,231 -> 4,470; warp
+// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,365 -> 4,496; warp
 // instructions 5.97e9 -> 3.33e9, DRAM 11.1 -> 0.9 GB (the tape stays in L2); 24
 // small problems, one gradient 245 -> 185.
 #pragma once
