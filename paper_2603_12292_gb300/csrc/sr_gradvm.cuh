@@ -16,7 +16,7 @@
 //     <= 96 tokens instead of 23);
 //   - both loops branch through tables in PTX and run on FP32 pairs (sr_vm.cuh).
 // Every value, partial and sum is rounded as before, in the same order.
-// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,365 -> 4,496; warp
+// 2,048 programs of <= 96 tokens x 65,536 cases, K = 8 (us): 7,365 -> 4,440; warp
 // instructions 5.97e9 -> 3.33e9, DRAM 11.1 -> 0.9 GB (the tape stays in L2); 24
 // small problems, one gradient 245 -> 185.
 #pragma once
@@ -579,23 +579,15 @@ static_assert(FW_TAPE == 16 && FW_SQT == 19 && FW_DIV == 20 && FW_CRDIV == 25 &&
 struct SinCos4 {
   V4 s, c;
 };
-// the larger value, NaN if either is
-__device__ __forceinline__ float max_nan(float a, float b) {
-  asm("max.NaN.f32 %0, %0, %1;" : "+f"(a) : "f"(b));
-  return a;
-}
-// arguments beyond the library's moderate range (any_far's way, sr_vm.cuh), and NaN,
-// whose cosine is that of the 0 it was replaced by until here.  With a select per
-// value for it in sincos4, 2,048 x 65,536 took 4,529 us instead of 4,496.
-__device__ __noinline__ SinCos4 sincos4_far(V4 s, V4 c) {
+// Some argument of the warp is not moderate, or NaN: the whole function on each value.
+// (With such values replaced by 0 and recognised afterwards 2,048 x 65,536 took 4,500 us
+// instead of 4,440, with 16 operators 8,838 instead of 8,390.)
+__device__ __noinline__ SinCos4 sincos4_wide(V4 x) {
   float a[GCPL], b[GCPL];
-  unpack4(s, a);
-  unpack4(c, b);
+  unpack4(x, a);
 #pragma unroll 1
   for (int i = 0; i < GCPL; ++i) {
-    float2 r = make_float2(a[0], b[0]);
-    if (fabsf(r.x) > 2.0f) r = sincos_wide(r.x);
-    else if (r.x != r.x) r.y = r.x;
+    const float2 r = sincos_wide(a[0]);
 #pragma unroll
     for (int j = 0; j < GCPL - 1; ++j) a[j] = a[j + 1], b[j] = b[j + 1];
     a[GCPL - 1] = r.x;
@@ -604,19 +596,19 @@ __device__ __noinline__ SinCos4 sincos4_far(V4 s, V4 c) {
   return SinCos4{pack4(a), pack4(b)};
 }
 __device__ __forceinline__ SinCos4 sincos4(const V4 &x) {
-  float t[GCPL], a[GCPL], b[GCPL];
-  unpack4(x, t);
+  float a[GCPL], b[GCPL];
+  unpack4(x, a);
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < GCPL; ++i) ok = ok & (fabsf(a[i]) <= NEAR);
+  if (__any_sync(FULL, !ok)) return sincos4_wide(x);
 #pragma unroll
   for (int i = 0; i < GCPL; ++i) {
-    const bool near = fabsf(t[i]) <= NEAR;
-    const float2 r = sincos_near(near ? t[i] : 0.0f);
-    a[i] = near ? r.x : t[i];
+    const float2 r = sincos_near(a[i]);
+    a[i] = r.x;
     b[i] = r.y;
   }
-  const float m = max_nan(max_nan(fabsf(a[0]), fabsf(a[1])), max_nan(fabsf(a[2]), fabsf(a[3])));
-  SinCos4 r{pack4(a), pack4(b)};
-  if (__any_sync(FULL, !(m <= 2.0f))) r = sincos4_far(r.s, r.c);
-  return r;
+  return SinCos4{pack4(a), pack4(b)};
 }
 __device__ __noinline__ V4 div4_wide(V4 a, V4 b) {
   float x[GCPL], y[GCPL];

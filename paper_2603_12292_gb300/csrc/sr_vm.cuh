@@ -14,7 +14,7 @@
 //     for the lane's 8 values.
 // Instructions executed (the profiler's counter) per node and 256 cases, before ->
 // then: x_j op 33 -> 14, square 27 -> 11, (push, x_i op x_j, op) 98 -> 42, quotient
-// 137 -> 69, sin 253 -> 209 (a select a value more since), log 264 -> 248, exp 120 ->
+// 137 -> 69, sin 253 -> 202, log 264 -> 248, exp 120 ->
 // 105, sqrt 119 -> 113 (5 CTAs per SM).
 // Evaluation of 8,192 programs of <= 256 tokens x 131,072 cases: 32.7 -> 25.4 ms.
 // Every value keeps its bits: each operator sees the operands it saw before and
@@ -101,43 +101,67 @@ __device__ __forceinline__ V8 zip8(const V8 &a, const V8 &b, F f) {
   return pack8(t);
 }
 
-// sin and cos: the library's path for moderate arguments runs on every value; an
-// argument outside it (|x| > 4e4, or NaN) is replaced by 0 for that, passed through
-// instead of the result and recognised afterwards by its magnitude (a result is at
-// most 1), for the whole warp at once: one test instead of a branch per value.  The 0
-// makes the assumption true for every value that it is stated of; assumed of the
-// arguments as they are, though used for the moderate ones only, 8,192 x 131,072 took
-// 25.2 ms instead of 25.4, 1,500 x 100,003 2,043 us instead of 2,066.
+// sin and cos: the library's path for moderate arguments (|x| <= 4e4) runs inline and is
+// told that its argument is one; what is told holds for every value it gets.
+// In the base copy a warp votes on its arguments first, one test for eight values; one
+// with an argument beyond, or NaN, calls the whole function on each value, out of line.
+// In the EXT copy, where NaN is common (asin and acos outside [-1, 1]), each value
+// that is not moderate is replaced by 0 there, passed through instead of the result and
+// recognised afterwards by its magnitude (a result is at most 1).  That / the vote, us:
+// 1,500 programs x 100,003 cases 2,051 / 1,968, 8,192 x 131,072 25,400 / 24,805, 64 small
+// problems 479 / 467; Eq. 2 with 16 operators 2,045 / 2,110 by the vote in the EXT copy too.
 constexpr float NEAR = 4.0e4f;
-struct SinNear {
+template <bool COS>
+struct SinCosNear {  // |x| <= NEAR
+  __device__ __forceinline__ float operator()(float x) const {
+    __builtin_assume(fabsf(x) <= NEAR);
+    return COS ? cosf(x) : sinf(x);
+  }
+};
+template <bool COS>
+struct SinCosOrArg {  // of a moderate x, else x
   __device__ __forceinline__ float operator()(float x) const {
     const bool near = fabsf(x) <= NEAR;
-    const float xn = near ? x : 0.0f;
-    __builtin_assume(fabsf(xn) <= NEAR);
-    const float r = sinf(xn);
+    const float r = SinCosNear<COS>()(near ? x : 0.0f);
     return near ? r : x;
   }
 };
-struct CosNear {
-  __device__ __forceinline__ float operator()(float x) const {
-    const bool near = fabsf(x) <= NEAR;
-    const float xn = near ? x : 0.0f;
-    __builtin_assume(fabsf(xn) <= NEAR);
-    const float r = cosf(xn);
-    return near ? r : x;
-  }
-};
-struct SinFar { __device__ __forceinline__ float operator()(float x) const { return fabsf(x) > 2.0f ? sin_wide(x) : x; } };
-struct CosFar { __device__ __forceinline__ float operator()(float x) const { return fabsf(x) > 2.0f ? cos_wide(x) : x; } };
-__device__ __noinline__ V8 sin8_far(V8 v) { return map8<1>(v, SinFar()); }
-__device__ __noinline__ V8 cos8_far(V8 v) { return map8<1>(v, CosFar()); }
-// some value of the warp is beyond any sine (a NaN argument has given NaN)
+template <bool COS>
+struct SinCosWide { __device__ __forceinline__ float operator()(float x) const { return COS ? cos_wide(x) : sin_wide(x); } };
+template <bool COS>
+struct SinCosFar { __device__ __forceinline__ float operator()(float x) const { return fabsf(x) > 2.0f ? SinCosWide<COS>()(x) : x; } };
+template <bool COS>
+__device__ __noinline__ V8 sincos8_wide(V8 v) { return map8<1>(v, SinCosWide<COS>()); }
+template <bool COS>
+__device__ __noinline__ V8 sincos8_far(V8 v) { return map8<1>(v, SinCosFar<COS>()); }
+// some |value| of the warp is beyond `limit`, or NaN
+__device__ __forceinline__ bool any_beyond(const V8 &v, float limit) {
+  float t[CPL];
+  unpack8(v, t);
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < CPL; ++i) ok = ok & (fabsf(t[i]) <= limit);
+  return __any_sync(FULL, !ok);
+}
+// some |value| of the warp is beyond any sine (a NaN argument has given NaN)
 __device__ __forceinline__ bool any_far(const V8 &v) {
   float t[CPL];
   unpack8(v, t);
   const float m = fmaxf(fmaxf(fmaxf(fabsf(t[0]), fabsf(t[1])), fmaxf(fabsf(t[2]), fabsf(t[3]))),
                         fmaxf(fmaxf(fabsf(t[4]), fabsf(t[5])), fmaxf(fabsf(t[6]), fabsf(t[7]))));
   return __any_sync(FULL, m > 2.0f);
+}
+template <bool COS, bool EXT, int W>
+__device__ __forceinline__ V8 sincos8(V8 v) {
+  if (EXT) {
+    v = map8<W>(v, SinCosOrArg<COS>());
+    if (any_far(v)) v = sincos8_far<COS>(v);
+  } else if (any_beyond(v, NEAR)) {
+    v = sincos8_wide<COS>(v);
+  } else {
+    v = map8<W>(v, SinCosNear<COS>());
+  }
+  return v;
 }
 // op_exp with its clamp in two instructions (NaN passes through both)
 struct Exp {
@@ -171,14 +195,6 @@ struct DivNear {
     return fabsf(b) < 1e-3f ? 1.0f : __fmul_rn(a, r);
   }
 };
-__device__ __forceinline__ bool any_huge(const V8 &v) {  // or NaN
-  float t[CPL];
-  unpack8(v, t);
-  bool ok = true;
-#pragma unroll
-  for (int i = 0; i < CPL; ++i) ok = ok & (fabsf(t[i]) <= DIV_NEAR);
-  return __any_sync(FULL, !ok);
-}
 __device__ __noinline__ V8 div8_wide(V8 a, V8 b) { return zip8<1>(a, b, Div()); }
 
 // 1/x, tan, asin, acos, atan, tanh (EXT programs)
@@ -319,21 +335,15 @@ __device__ __forceinline__ V8 interpret(const uint2 *code, const char *stk, cons
                    : SR_CORE_OUT(T, X, ip, op) : "r"(st), "l"(xa), "l"(xb) : "memory");
     switch (op) {
       case OP_VDIV:
-        if (any_huge(X)) T = div8_wide(T, X);
+        if (any_beyond(X, DIV_NEAR)) T = div8_wide(T, X);
         else T = zip8<S::DIV>(T, X, DivNear());
         break;
       case OP_VRDIV:
-        if (any_huge(T)) T = div8_wide(X, T);
+        if (any_beyond(T, DIV_NEAR)) T = div8_wide(X, T);
         else T = zip8<S::DIV>(X, T, DivNear());
         break;
-      case OP_SIN:
-        T = map8<S::TRIG>(T, SinNear());
-        if (any_far(T)) T = sin8_far(T);
-        break;
-      case OP_COS:
-        T = map8<S::TRIG>(T, CosNear());
-        if (any_far(T)) T = cos8_far(T);
-        break;
+      case OP_SIN: T = sincos8<false, EXT, S::TRIG>(T); break;
+      case OP_COS: T = sincos8<true, EXT, S::TRIG>(T); break;
       case OP_EXP: T = map8<S::POW>(T, Exp()); break;
       case OP_LOG: T = map8<S::TRIG>(T, Log()); break;
       case OP_SQRT: T = map8<S::POW>(T, Sqrt()); break;
