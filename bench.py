@@ -48,25 +48,25 @@ KERNEL_SOURCES = {
 # workload, and for another size only where it grows with the units (scale).
 KERNEL_NCU = {
     # eval_kernel<MODE_BOTH> on the headline workload, inputs read once
-    "paper": {"workload": "paper-4096x100k", "dram_bytes": 174.698e6 + 18.331e6, "units": None,
-              "issue_active": 0.829, "scale": False, "sources": "eval",
-              "capture": "profiles/eval_kernel_paper-4096x100k.md", "src": "d5cc61786de98123"},
+    "paper": {"workload": "paper-4096x100k", "dram_bytes": 174.640e6 + 17.675e6, "units": None,
+              "issue_active": 0.823, "scale": False, "sources": "eval",
+              "capture": "profiles/eval_kernel_paper-4096x100k.md", "src": "26fab55eb25960cb"},
     # grad_kernel: the write-back of the tape's lines grows with the units
-    "grad": {"workload": "adjoint-2048x131072", "dram_bytes": 0.018e9 + 1.686e9, "units": 1.3324e10,
-             "issue_active": 0.636, "scale": True, "sources": "grad",
-             "capture": "profiles/grad_kernel_adjoint-2048x131072.md", "src": "a8c38c6111c1ee14"},
+    "grad": {"workload": "adjoint-2048x131072", "dram_bytes": 20.376e6 + 1686.692e6, "units": 1.3324e10,
+             "issue_active": 0.640, "scale": True, "sources": "grad",
+             "capture": "profiles/grad_kernel_adjoint-2048x131072.md", "src": "6224e98696248eca"},
     # eval_kernel<R4>: inputs read once (L2-resident), at the full size
-    "beagle": {"workload": "beagle-4096x100k", "dram_bytes": 171.694e6 + 15.975e6, "units": 2.3977e10,
-               "issue_active": 0.823, "scale": False, "sources": "eval",
-               "capture": "profiles/eval_kernel_r4_beagle-4096x100k.md", "src": "d5cc61786de98123"},
+    "beagle": {"workload": "beagle-4096x100k", "dram_bytes": 171.372e6 + 15.990e6, "units": 2.3977e10,
+               "issue_active": 0.829, "scale": False, "sources": "eval",
+               "capture": "profiles/eval_kernel_r4_beagle-4096x100k.md", "src": "26fab55eb25960cb"},
     # eval_batched_kernel: the first 8 problems; inputs read once
-    "batched": {"workload": "batched-8", "dram_bytes": 2060.8e6 + 174.64e6, "units": 4.0723e11,
-                "issue_active": 0.808, "scale": False, "sources": "eval",
-                "capture": "profiles/eval_batched_kernel_batched-8.md", "src": "d5cc61786de98123"},
+    "batched": {"workload": "batched-8", "dram_bytes": 1956.351e6 + 172.981e6, "units": 4.0723e11,
+                "issue_active": 0.799, "scale": False, "sources": "eval",
+                "capture": "profiles/eval_batched_kernel_batched-8.md", "src": "26fab55eb25960cb"},
     # eval_kernel<CORR> at Lmax 256: inputs read once
-    "large": {"workload": "large-16384x131072", "dram_bytes": 518.4e6 + 82.126e6, "units": 2.5087e11,
-              "issue_active": 0.795, "scale": False, "sources": "eval",
-              "capture": "profiles/eval_kernel_corr_large-16384x131072.md", "src": "d5cc61786de98123"},
+    "large": {"workload": "large-16384x131072", "dram_bytes": 511.533e6 + 80.602e6, "units": 2.5087e11,
+              "issue_active": 0.784, "scale": False, "sources": "eval",
+              "capture": "profiles/eval_kernel_corr_large-16384x131072.md", "src": "26fab55eb25960cb"},
 }
 
 
